@@ -62,12 +62,14 @@ k_mlp(const double *feat, const float *w, int F, int H, int K, int time_head, in
     __syncthreads();
     for (int j = t; j < H; j += blockDim.x) {
         float a = b1[j];
+#pragma unroll 10
         for (int k = 0; k < F; ++k) a = fmaf(W1[j * F + k], z[k], a);
         hid[j] = a > 0.f ? a : 0.f;
     }
     __syncthreads();
     for (int o = t; o < K; o += blockDim.x) {
         float a = b2[o];
+#pragma unroll 16  // the weights' loads go out together; the sum keeps its order
         for (int j = 0; j < H; ++j) a = fmaf(W2[o * H + j], hid[j], a);
         lg[o] = a;
         if (logits) logits[o] = a;
@@ -75,6 +77,7 @@ k_mlp(const double *feat, const float *w, int F, int H, int K, int time_head, in
     if (time_head && logt) {
         for (int o = t; o <= K; o += blockDim.x) {
             float a = b3[o];
+#pragma unroll 16
             for (int j = 0; j < H; ++j) a = fmaf(W3[o * H + j], hid[j], a);
             logt[o] = a;
         }
@@ -82,8 +85,13 @@ k_mlp(const double *feat, const float *w, int F, int H, int K, int time_head, in
     __syncthreads();
     if (t == 0) {
         int best = 0;
+        float top = lg[0];
+#pragma unroll 8
         for (int o = 1; o < K; ++o)
-            if (lg[o] > lg[best]) best = o;
+            if (lg[o] > top) {
+                top = lg[o];
+                best = o;
+            }
         *choice = best;
     }
 }
