@@ -488,14 +488,18 @@ SPMV_API int spmv_select_runtime(spmv_handle h, int64_t expected_runs,
  *     alpha = rho_k / (p_k.q); x += alpha p_k; r -= alpha q;
  *     p_{k+1} = r_{k+1} + (rho_{k+1} / rho_k) p_k.
  * A must be square and symmetric positive definite; every product runs in
- * the handle's current format and configuration.
+ * the handle's current format and configuration, except that small systems
+ * (up to 32768 rows, rows of up to 64 entries, 393216 entries) are solved
+ * from the handle's CSR arrays by one thread-block cluster that keeps the
+ * vectors on chip.
  *
  * d_b: device, m entries (double for SPMV_F64 handles, float otherwise),
  *      read only.  d_x: device, same type; in: x_0, out: the last iterate.
  * d_rho: NULL, or device double[maxit + 1] receiving rho_0 .. rho_iterations.
  * Dot products accumulate in fp64 in a fixed order (repeat calls are
  * bit-identical).  The whole loop is one CUDA graph whose WHILE node the
- * device stops: no host round trip per iteration.  The handle keeps the
+ * device stops (small systems: one kernel): no host round trip per
+ * iteration.  The handle keeps the
  * graph and three m-vectors of scratch for the next call with the same
  * (d_b, d_x, tol, maxit); spmv_set_config and spmv_destroy release them.
  * Synchronises `stream`, then fills *out.
