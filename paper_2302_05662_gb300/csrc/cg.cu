@@ -693,9 +693,15 @@ struct ClusterLaunch {
 // 5-point fp64 1024 rows 5.6 / 19.5, 4096 5.8 / 20.0, 32,700 12.1 / 22.1;
 // 27-point fp64 8000 rows (195K entries, staged) 9.8 / 23.6, 13,824 (343K,
 // read in place) 18.2 / 23.6, 19,683 (507K) 29.0 / 24.7, fp32 23.6 / 23.4.
-// A row is one thread's serial work, hence the limit on its length.
+// A row is one thread's serial work, hence the limit on its length.  It is
+// summed in column order, as the formats with one lane per row sum it, so only
+// those take this form: a handle set to another format keeps that format's
+// products.
 bool cluster_fits(const spmv_matrix *h, int *ctas, int *shift, int *cap) {
-    if (h->npanels > 0 || h->m > (int64_t)CL_MAX_CTAS * CL_THREADS * CL_MAX_RPT || h->max_row > CL_MAX_ROW ||
+    const int fmt = h->cfg.format;
+    const bool lane_rows = fmt == SPMV_FMT_ELL || fmt == SPMV_FMT_SELL || (fmt == SPMV_FMT_HYB && h->hyb_nnz == 0) ||
+                           (fmt == SPMV_FMT_CSR && h->cfg.threads_per_row == 1 && !csr_uneven(h, 1));
+    if (!lane_rows || h->npanels > 0 || h->m > (int64_t)CL_MAX_CTAS * CL_THREADS * CL_MAX_RPT || h->max_row > CL_MAX_ROW ||
         h->nnz > CL_MAX_NNZ)
         return false;
     int sh = 8, n = 1;

@@ -56,7 +56,7 @@ def test_rows_around_the_cluster_sizes(oracle, n):
 @pytest.mark.parametrize("n,w", [(700, 31), (700, 32), (4096, 31), (6000, 31), (6400, 31)])
 def test_row_lengths_and_entry_limits(oracle, n, w):
     """63 and 65 entries a row; rows staged (4096) and read in place (6000); 403,000 entries."""
-    check(oracle, band(n, w), None)
+    check(oracle, band(n, w), B.make_config(format=B.FMT_ELL))
 
 
 @pytest.mark.parametrize("fmt", [n for n, _ in SWEEP_VARIANTS])
