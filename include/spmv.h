@@ -114,7 +114,8 @@ typedef enum {
  *                     1/2/4/8 (default 1).  Ignored by ELL, COO, HYB and
  *                     SELL (one lane per row).
  *   unroll            1, 2 or 4 (8 also for ELL, HYB and SELL): loads in
- *                     flight per lane (ELL, SELL, CSR) or items per lane / 4
+ *                     flight per lane (ELL, SELL, CSR; fixed for CSR with
+ *                     1 or 2 lanes on very uneven rows) or items per lane / 4
  *                     (COO, HYB tail, split CSR; at most 16 items).  0 =
  *                     default: ELL and HYB 2 with fp64 values, 4 with
  *                     fp32/bf16; SELL 8 (1 with fp64 values in the
@@ -489,9 +490,10 @@ SPMV_API int spmv_select_runtime(spmv_handle h, int64_t expected_runs,
  *     p_{k+1} = r_{k+1} + (rho_{k+1} / rho_k) p_k.
  * A must be square and symmetric positive definite; every product runs in
  * the handle's current format and configuration, except that small systems
- * (up to 32768 rows, rows of up to 64 entries, 393216 entries) are solved
- * from the handle's CSR arrays by one thread-block cluster that keeps the
- * vectors on chip.
+ * (up to 32768 rows, rows of up to 64 entries, 393216 entries) in a format
+ * with one lane per row (ELL, SELL, HYB without a tail, CSR with one thread
+ * per row) are solved from the handle's CSR arrays, rows summed in the same
+ * order, by one thread-block cluster that keeps the vectors on chip.
  *
  * d_b: device, m entries (double for SPMV_F64 handles, float otherwise),
  *      read only.  d_x: device, same type; in: x_0, out: the last iterate.

@@ -108,13 +108,23 @@ __global__ void k_expand_rows(const int *rowptr, int64_t m, int64_t nnz, int *ro
         rows[k] = row_of(rowptr, m, k);
 }
 
-__global__ void k_max_row(const int *rowptr, int64_t m, int *out) {
+// longest row, and the sum over groups of 32 rows of the group's longest row
+// (counted up to 512 entries): what a warp with a lane per row waits for
+__global__ void k_max_row(const int *rowptr, int64_t m, int *out, unsigned long long *group_sum) {
     int best = 0;
+    unsigned long long sum = 0;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m; r += stride)
-        best = max(best, rowptr[r + 1] - rowptr[r]);
+    const int64_t mr = (m + 31) / 32 * 32;
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < mr; r += stride) {
+        const int len = r < m ? rowptr[r + 1] - rowptr[r] : 0;
+        best = max(best, len);
+        sum += (unsigned)__reduce_max_sync(FULL, min(len, 512));
+    }
     best = __reduce_max_sync(FULL, best);
-    if ((threadIdx.x & 31) == 0) atomicMax(out, best);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(out, best);
+        atomicAdd(group_sum, sum);
+    }
 }
 
 // consecutive stored entries whose columns are consecutive (col[k] ==
@@ -974,16 +984,17 @@ int build_csr(spmv_matrix *h, const int32_t *d_rows, const int32_t *d_cols, cons
         k_rowptr_from_sorted<<<grid1d(m + 1, 256), 256, 0, s>>>(urows.p, nu, m, h->rowptr);
         SPMV_CUDA_TRY(cudaGetLastError());
     }
-    Tmp<unsigned long long> mx;   // [0]: longest row, [1]: contiguous pairs
-    SPMV_TRY(mx.alloc(2, s));
-    SPMV_CUDA_TRY(cudaMemsetAsync(mx.p, 0, 2 * sizeof(unsigned long long), s));
-    if (m > 0) k_max_row<<<grid1d(m, 256), 256, 0, s>>>(h->rowptr, m, reinterpret_cast<int *>(mx.p));
+    Tmp<unsigned long long> mx;   // [0]: longest row, [1]: contiguous pairs, [2]: longest rows of 32-row groups
+    SPMV_TRY(mx.alloc(3, s));
+    SPMV_CUDA_TRY(cudaMemsetAsync(mx.p, 0, 3 * sizeof(unsigned long long), s));
+    if (m > 0) k_max_row<<<grid1d(m, 256), 256, 0, s>>>(h->rowptr, m, reinterpret_cast<int *>(mx.p), mx.p + 2);
     if (h->nnz > 1) k_contiguous_pairs<<<grid1d(h->nnz, 256), 256, 0, s>>>(h->colidx, h->nnz, mx.p + 1);
     SPMV_CUDA_TRY(cudaGetLastError());
-    unsigned long long hmx[2] = {0, 0};
+    unsigned long long hmx[3] = {0, 0, 0};
     SPMV_CUDA_TRY(cudaMemcpyAsync(hmx, mx.p, sizeof(hmx), cudaMemcpyDeviceToHost, s));
     SPMV_CUDA_TRY(cudaStreamSynchronize(s));
     h->max_row = (int64_t)(hmx[0] & 0xffffffffull);
+    h->group_max = m > 0 ? (double)hmx[2] / (double)((m + 31) / 32) : 0.0;
     h->contig = h->nnz > 1 ? (double)hmx[1] / (double)(h->nnz - 1) : 0.0;
     return SPMV_OK;
 }
@@ -1411,9 +1422,12 @@ int pack_format(spmv_matrix *h, const spmv_config &cfg, cudaStream_t s) {
             if (cfg.hyb_ell_width == 0) SPMV_TRY(ensure_seg_scratch(h, items, SEG_MERGE, s));
             else SPMV_TRY(ensure_seg_scratch(h, cfg.hyb_ell_width / 32, SEG_TILES, s));
         } else {
-            // rows needing more than 32 steps of their lane group go to whole blocks
-            const int64_t thr = std::max<int64_t>(512, 32LL * cfg.threads_per_row * cfg.unroll);
-            SPMV_TRY(build_long_rows(h, h->rowptr, h->m, thr, 4096, 1, s));
+            // rows needing more than 32 steps of their lane group go to whole blocks (uneven rows
+            // with one or two lanes: to warps)
+            const bool uneven = csr_uneven(h, cfg.threads_per_row);
+            const int64_t thr =
+                uneven ? CSR_WARP_ROW : std::max<int64_t>(512, 32LL * cfg.threads_per_row * cfg.unroll);
+            SPMV_TRY(build_long_rows(h, h->rowptr, h->m, thr, uneven ? CSR_SEG_LEN : 4096, 1, s));
         }
         break;
     case SPMV_FMT_ELL: {

@@ -307,6 +307,7 @@ struct CgPlan;
 struct spmv_matrix {
     int64_t m = 0, n = 0, nnz = 0, max_row = 0;
     double contig = 0.0;  // fraction of consecutive stored entries with consecutive columns
+    double group_max = 0.0;  // mean over groups of 32 rows of the longest row (up to 512)
     int32_t vt = SPMV_F64;
     spmv_config cfg{};
     spmv_config packed_req{};  // configuration the current packs were built for
@@ -406,6 +407,24 @@ int run_kernels_f32(int kind, const spmv_matrix *h, double alpha, const void *x,
                     cudaStream_t s);
 int run_kernels_bf16(int kind, const spmv_matrix *h, double alpha, const void *x, double beta, void *y,
                      cudaStream_t s);
+
+// Vector CSR with one or two lanes per row runs as k_csr_skew where the
+// longest of 32 neighbouring rows is, on average, over two mean rows and 16
+// entries more: a warp of k_csr_vector waits for it.  (Random rows of mean 2
+// to 31 stay well below the line, R-MAT above it; a few long rows alone do not
+// reach it: even rows are faster in k_csr_vector, 27-point stencil 142 against
+// 274 us.)  Rows of up to CSR_MEDIUM_ROW entries then take a lane, up to
+// CSR_WARP_ROW eight lanes, longer ones a warp for each CSR_SEG_LEN entries.
+// R-MAT scale 20 fp64 / scale 14 fp64, us: 127.6 / 39.2 when only rows over
+// 512 took warps, 107.8 / 15.3 with 128, 111.7 / 16.0 with 64; segments of 512
+// entries 113.1, of 2048 106.6 (but scale 17: 22.8 against 20.1); medium rows
+// from 8, 16, 24, 32: 110.1, 108.8, 107.8, 108.6.
+constexpr int CSR_MEDIUM_ROW = 24, CSR_WARP_ROW = 128, CSR_SEG_LEN = 1024;
+inline bool csr_uneven(const spmv_matrix *h, int threads_per_row) {
+    if (threads_per_row != 1 && threads_per_row != 2) return false;
+    const double mean = h->m > 0 ? (double)h->nnz / (double)h->m : 0.0;
+    return h->group_max > 2.0 * mean + 16.0;
+}
 
 // default lanes per row of vector CSR for this matrix (api.cu)
 int default_tpr(const spmv_matrix *h);

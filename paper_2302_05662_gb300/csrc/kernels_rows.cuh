@@ -218,6 +218,119 @@ k_csr_long(int64_t nseg, const int *__restrict__ seg_row, const int *__restrict_
 }
 
 // ---------------------------------------------------------------------------
+// Vector CSR with one or two lanes per row on uneven rows.  What bounds
+// k_csr_vector there is balance: a warp lasts as long as the longest of its
+// 32 rows (up to 512 entries one after the other), and the longer rows wait
+// for all others in a kernel of their own.  Here a warp takes 32 rows; those
+// of up to `medium` entries are summed by a lane each, longer ones by eight
+// lanes, and rows over long_threshold are cut into segments of one warp.
+// One group of rows or one segment per warp and as many blocks as that takes:
+// the block scheduler balances what a fixed share per resident warp cannot.
+// Segments come first in the grid, so that the longest work starts first.
+// R-MAT scale 20, fp64, default configuration: 353 us as k_csr_vector and
+// k_csr_long, 108 here; fp32 235 and 65.
+// ---------------------------------------------------------------------------
+// The rows of `mask` (bit l: the warp's row l, at entries [s, e) of lane l)
+// summed by eight lanes each, four rows at a time, U gathers in flight per
+// lane: three shuffle adds for four rows, where a warp per row makes five for
+// one (fp64 adds are the scarce instruction here).
+template <typename V, typename T, int U>
+__device__ __forceinline__ void csr_medium_rows(unsigned mask, int my_s, int my_e, int64_t base,
+                                                const int *__restrict__ colidx, const V *__restrict__ vals,
+                                                const T *__restrict__ x, T *__restrict__ y, const Epi<T> &ep) {
+    const int lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3;
+#pragma unroll 1
+    while (mask) {
+        unsigned mine = mask;  // group g takes the g-th lowest bit
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            if (i < grp) mine &= mine - 1;
+        const int src = mine ? __ffs(mine) - 1 : 0;
+        const int s = __shfl_sync(FULLMASK, my_s, src);
+        const int end = __shfl_sync(FULLMASK, my_e, src);  // every lane takes part
+        const int e = mine ? end : s;
+        T acc = T(0);
+        for (int k = s + sub; k < e; k += 8 * U) {
+            int c[U];
+            T v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int kk = k + 8 * u;
+                c[u] = kk < e ? ld_s(colidx + kk) : -1;
+                v[u] = kk < e ? ld_val(vals + kk) : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (c[u] >= 0) acc = fma(v[u], ld_x(x, c[u]), acc);
+        }
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) acc += __shfl_down_sync(FULLMASK, acc, off, 8);
+        if (sub == 0 && mine) ep.store(y, base + src, acc);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) mask &= mask - 1;  // 0 stays 0
+    }
+}
+
+// Segments of long rows (LongRows): one warp each, joined through the
+// partials in segment order.
+struct LongSegs {
+    int64_t n;
+    const int *row, *begin, *end, *c0, *c1;
+};
+
+template <typename V, typename T, int U>
+__device__ __forceinline__ void csr_long_segment(int64_t k, const LongSegs &L, const int *__restrict__ colidx,
+                                                 const V *__restrict__ vals, const T *__restrict__ x,
+                                                 T *__restrict__ y, const Epi<T> &ep, const PartialsT<T> &P) {
+    const int lane = threadIdx.x & 31;
+    const int b = __ldg(L.begin + k), e = __ldg(L.end + k);
+    T acc = T(0);
+    for (int i = b + lane; i < e; i += 32 * U) {
+        int c[U];
+        T v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int ii = i + 32 * u;
+            c[u] = ii < e ? ld_s(colidx + ii) : -1;
+            v[u] = ii < e ? ld_val(vals + ii) : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (c[u] >= 0) acc = fma(v[u], ld_x(x, c[u]), acc);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(FULLMASK, acc, off);
+    if (lane == 0) {
+        const int64_t c0 = __ldg(L.c0 + k), c1 = __ldg(L.c1 + k);
+        T total = acc;
+        if (c0 == c1 || join_partial<T>(k, c0, c1, 0, acc, P, &total)) ep.store(y, __ldg(L.row + k), total);
+    }
+}
+
+template <typename V, typename T, int REGCAP>
+__global__ void __launch_bounds__(1024) __maxnreg__(REGCAP)
+k_csr_skew(int64_t m, const int *__restrict__ rowptr, const int *__restrict__ colidx, const V *__restrict__ vals,
+           const T *__restrict__ x, T *__restrict__ y, T alpha, T beta, int long_threshold, int medium,
+           const LongSegs L, const PartialsT<T> P) {
+    const Epi<T> ep(alpha, beta);
+    constexpr int U = REGCAP <= 32 ? 2 : 4;
+    const int lane = threadIdx.x & 31;
+    const int64_t unit = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (unit < L.n) {
+        csr_long_segment<V, T, U>(unit, L, colidx, vals, x, y, ep, P);
+        return;
+    }
+    const int64_t row = (unit - L.n) * 32 + lane;
+    const int s = row < m ? __ldg(rowptr + row) : 0;
+    const int e = row < m ? __ldg(rowptr + row + 1) : 0;
+    const int len = e - s;
+    if (row < m && len <= medium) ep.store(y, row, csr_lane_range<V, T, (REGCAP <= 32 ? 1 : 2), 4>(s, e, colidx, vals, x));
+    __syncwarp();
+    const unsigned mask = __ballot_sync(FULLMASK, len > medium && len <= long_threshold);
+    if (mask) csr_medium_rows<V, T, U>(mask, s, e, row - lane, colidx, vals, x, y, ep);
+}
+
+// ---------------------------------------------------------------------------
 // ELL, column-major [width][pitch] (Section 2.3: m x max_nnz Data and Column
 // Index matrices).  Padding has column -1 and rows are left-packed, so a
 // thread stops at its first padding slot and reads no padding values.

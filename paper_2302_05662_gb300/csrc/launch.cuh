@@ -53,6 +53,23 @@ int launch_bsr_long(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, cud
 }
 
 // ------------------------------- CSR vector --------------------------------
+template <typename V, typename T, int RC>
+int launch_csr_skew(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, cudaStream_t s) {
+    auto kern = k_csr_skew<V, T, RC>;
+    // small blocks: one is done when its slowest warp is (R-MAT scale 20: 108 us
+    // with 128 threads, 115 with 256)
+    const int tpb = std::min(128, h->cfg.threads_per_block);
+    SPMV_TRY(apply_carveout((const void *)kern, h->cfg.carveout));
+    const LongRows &L = h->lng;
+    const int64_t units = L.nseg + (h->m + 31) / 32, wpb = tpb / 32;
+    const int thr = L.nseg > 0 ? (int)L.threshold : 0x7fffffff;
+    kern<<<(unsigned)((units + wpb - 1) / wpb), tpb, 0, s>>>(
+        h->m, h->rowptr, h->colidx, (const V *)h->vals, x, y, alpha, beta, thr, CSR_MEDIUM_ROW,
+        LongSegs{L.nseg, L.seg_row, L.seg_begin, L.seg_end, L.seg_c0, L.seg_c1}, PartialsT<T>::of(L.part));
+    SPMV_LAUNCH_CHECK();
+    return SPMV_OK;
+}
+
 template <typename V, typename T, int TPR, int U, int RC, int GW>
 int launch_csr_vector(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, cudaStream_t s) {
     auto kern = k_csr_vector<V, T, TPR, U, RC, GW>;
@@ -71,6 +88,9 @@ int launch_csr_vector(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, c
 template <typename V, typename T, int TPR, int U>
 int csr_vector_rc(const spmv_matrix *h, T a, const T *x, T b, T *y, cudaStream_t s) {
     if constexpr (TPR <= 2) {
+        if (csr_uneven(h, h->cfg.threads_per_row))
+            return h->cfg.regcap == 32 ? launch_csr_skew<V, T, 32>(h, a, x, b, y, s)
+                                       : launch_csr_skew<V, T, 64>(h, a, x, b, y, s);
         if (h->cfg.bsr_block == 8)
             return h->cfg.regcap == 32 ? launch_csr_vector<V, T, TPR, U, 32, 8>(h, a, x, b, y, s)
                                        : launch_csr_vector<V, T, TPR, U, 64, 8>(h, a, x, b, y, s);
