@@ -48,6 +48,12 @@ int dalloc_bytes(void **p, size_t bytes) {
     return SPMV_OK;
 }
 
+// The CSR arrays are allocated CSR_PAD entries longer than needed: the
+// staged tile kernel copies whole multiples of 8 column/value entries and
+// 16-byte windows of row pointers, so the last tile may read up to 7 entries
+// past nnz and 3 past m (never used).
+constexpr size_t CSR_PAD = 8;
+
 inline int bits_for(int64_t count) {  // bits to hold 0 .. count-1
     int b = 0;
     while ((int64_t(1) << b) < count) ++b;
@@ -58,25 +64,86 @@ inline unsigned grid1d(int64_t work, int threads, int cap = 152 * 32) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(g, cap));
 }
 
+// sums, maxima and bitwise ors of a block end in one atomic each: an atomic
+// per warp on one word held these passes up (R-MAT, 8.4M triplets: 45, 29 and
+// 22 us for check, contiguous pairs and longest row; 30, 9 and 3.5 now)
+__device__ __forceinline__ void block_add(unsigned v, unsigned long long *out) {
+    __shared__ unsigned s_v;
+    if (threadIdx.x == 0) s_v = 0;
+    __syncthreads();
+    v = __reduce_add_sync(FULL, v);
+    if ((threadIdx.x & 31) == 0 && v) atomicAdd(&s_v, v);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_v) atomicAdd(out, (unsigned long long)s_v);
+}
+
 // ---------------------------------------------------------------------------
 // validation: bit 0 = index out of range, bit 1 = not sorted by (row, col),
-// bit 2 = a repeated (row, col) pair
+// bit 2 = a repeated (row, col) pair, bit 3 = over ROW_GAP empty rows in a row.
+// The same pass forms what an ordered list needs besides: the row pointers
+// (each written at the entry that opens its row; not across a gap of bit 3)
+// and the number of consecutive entries with consecutive columns (a pair
+// across a row boundary counts too; the statistic only steers a layout
+// default).  An unordered list leaves both meaningless.
 // ---------------------------------------------------------------------------
-__global__ void k_check_triplets(const int *rows, const int *cols, int64_t nnz, int64_t m,
-                                 int64_t n, unsigned *flags) {
-    unsigned f = 0;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += stride) {
-        int r = rows[i], c = cols[i];
-        if (r < 0 || r >= m || c < 0 || c >= n) f |= 1u;
-        if (i + 1 < nnz) {
-            int r2 = rows[i + 1], c2 = cols[i + 1];
-            if (r2 < r || (r2 == r && c2 < c)) f |= 2u;
-            else if (r2 == r && c2 == c) f |= 4u;
+constexpr int ROW_GAP = 32, CHECK_STEPS = 8;
+
+__global__ void __launch_bounds__(256) k_check_triplets(const int *__restrict__ rows, const int *__restrict__ cols,
+                                                        int64_t nnz, int64_t m, int64_t n, unsigned *flags, int *rowptr,
+                                                        unsigned long long *contiguous) {
+    unsigned f = 0, cnt = 0;
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t stride = (((int64_t)gridDim.x * blockDim.x) >> 5) * (32 * CHECK_STEPS);
+    const unsigned mu = (unsigned)m, nu = (unsigned)n;  // below 2^31: one unsigned comparison checks both ends
+    // rows (r, r2] start at entry i
+    auto open_rows = [&](int r, int r2, int64_t i) {
+        if (r2 == r + 1) rowptr[r2] = (int)i;
+        else if (r2 - r > ROW_GAP) f |= 8u;
+        else
+            for (int q = r + 1; q <= r2; ++q) rowptr[q] = (int)i;
+    };
+    // a warp takes 32 CHECK_STEPS consecutive entries; an entry's successor is the next lane's
+    for (int64_t w0 = warp * (32 * CHECK_STEPS); w0 < nnz; w0 += stride) {
+        int r[CHECK_STEPS + 1], c[CHECK_STEPS + 1];
+        const int left = (int)(nnz - w0 < 32 * CHECK_STEPS + 1 ? nnz - w0 : 32 * CHECK_STEPS + 1);  // entries from w0 on
+        const int *rp = rows + w0 + lane, *cp = cols + w0 + lane;
+#pragma unroll
+        for (int j = 0; j <= CHECK_STEPS; ++j) {
+            const bool read = (j < CHECK_STEPS || lane == 0) && 32 * j + lane < left;
+            r[j] = read ? __ldg(rp + 32 * j) : 0;
+            c[j] = read ? __ldg(cp + 32 * j) : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < CHECK_STEPS; ++j) {
+            const int ru = __shfl_down_sync(FULL, r[j], 1), cu = __shfl_down_sync(FULL, c[j], 1);
+            const int rn = __shfl_sync(FULL, r[j + 1], 0), cn = __shfl_sync(FULL, c[j + 1], 0);
+            const int r2 = lane == 31 ? rn : ru, c2 = lane == 31 ? cn : cu;
+            if (32 * j + lane < left) {
+                const bool more = 32 * j + lane + 1 < left, in = (unsigned)r[j] < mu;
+                if (!in || (unsigned)c[j] >= nu) f |= 1u;
+                if (more) {
+                    if (r2 < r[j] || (r2 == r[j] && c2 < c[j])) f |= 2u;
+                    else if (r2 == r[j] && c2 == c[j]) f |= 4u;
+                    cnt += c2 == c[j] + 1;
+                }
+                if (rowptr && in && (r2 != r[j] || !more || (j == 0 && lane == 0))) {
+                    const int64_t i = w0 + 32 * j + lane;
+                    if (i == 0) open_rows(-1, r[j], 0);
+                    const unsigned next = more ? (unsigned)r2 : mu;
+                    if (next <= mu && (int)next > r[j]) open_rows(r[j], (int)next, i + 1);
+                }
+            }
         }
     }
+    __shared__ unsigned s_f;
+    if (threadIdx.x == 0) s_f = 0;
+    __syncthreads();
     f = __reduce_or_sync(FULL, f);
-    if ((threadIdx.x & 31) == 0 && f) atomicOr(flags, f);
+    if ((threadIdx.x & 31) == 0 && f) atomicOr(&s_f, f);
+    if (contiguous) block_add(cnt, contiguous);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_f) atomicOr(flags, s_f);
 }
 
 // rowptr[r] = first position whose row is >= r, over rows sorted ascending
@@ -110,9 +177,10 @@ __global__ void k_expand_rows(const int *rowptr, int64_t m, int64_t nnz, int *ro
 
 // longest row, and the sum over groups of 32 rows of the group's longest row
 // (counted up to 512 entries): what a warp with a lane per row waits for
-__global__ void k_max_row(const int *rowptr, int64_t m, int *out, unsigned long long *group_sum) {
+__global__ void __launch_bounds__(1024) k_max_row(const int *rowptr, int64_t m, unsigned long long *longest,
+                                                  unsigned long long *group_sum) {
     int best = 0;
-    unsigned long long sum = 0;
+    unsigned sum = 0;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t mr = (m + 31) / 32 * 32;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < mr; r += stride) {
@@ -120,23 +188,24 @@ __global__ void k_max_row(const int *rowptr, int64_t m, int *out, unsigned long 
         best = max(best, len);
         sum += (unsigned)__reduce_max_sync(FULL, min(len, 512));
     }
+    __shared__ int s_best;
+    if (threadIdx.x == 0) s_best = 0;
+    __syncthreads();
     best = __reduce_max_sync(FULL, best);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(out, best);
-        atomicAdd(group_sum, sum);
-    }
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_best, best);
+    block_add((threadIdx.x & 31) == 0 ? sum : 0u, group_sum);
+    if (threadIdx.x == 0) atomicMax(longest, (unsigned long long)s_best);
 }
 
-// consecutive stored entries whose columns are consecutive (col[k] ==
-// col[k-1] + 1): the column contiguity of the rows (a pair across a row
-// boundary can count too; the statistic only steers a layout default)
-__global__ void k_contiguous_pairs(const int *colidx, int64_t nnz, unsigned long long *out) {
-    unsigned long long cnt = 0;
+// consecutive stored entries whose columns are consecutive (as k_check_triplets counts them)
+__global__ void __launch_bounds__(256) k_contiguous_pairs(const int *__restrict__ colidx, int64_t nnz,
+                                                          unsigned long long *out) {
+    unsigned cnt = 0;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll 4
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x + 1; k < nnz; k += stride)
-        cnt += colidx[k] == colidx[k - 1] + 1;
-    cnt = __reduce_add_sync(FULL, (unsigned)cnt);
-    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(out, cnt);
+        cnt += __ldg(colidx + k) == __ldg(colidx + k - 1) + 1;
+    block_add(cnt, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -190,22 +259,29 @@ __global__ void __launch_bounds__(SC_THREADS) k_scan_reduce(const int *in, int64
     }
 }
 
-// single block: exclusive scan of nb tile sums in place
+// single block: exclusive scan of nb tile sums in place, their total in
+// sums[nb]
 __global__ void __launch_bounds__(SC_THREADS) k_scan_sums(int *sums, int64_t nb) {
-    __shared__ int carry_s;
     __shared__ int total_s;
-    if (threadIdx.x == 0) carry_s = 0;
-    __syncthreads();
-    for (int64_t base = 0; base < nb; base += SC_THREADS) {
-        int64_t i = base + threadIdx.x;
-        int v = i < nb ? sums[i] : 0;
-        int ex = block_exclusive_scan(v, &total_s);
-        int carry = carry_s;
-        if (i < nb) sums[i] = ex + carry;
-        __syncthreads();
-        if (threadIdx.x == 0) carry_s = carry + total_s;
+    int carry = 0;
+    for (int64_t base = 0; base < nb; base += SC_TILE) {
+        const int64_t at = base + (int64_t)threadIdx.x * SC_ITEMS;
+        int v[SC_ITEMS], t = 0;
+#pragma unroll
+        for (int j = 0; j < SC_ITEMS; ++j) {
+            v[j] = at + j < nb ? sums[at + j] : 0;
+            t += v[j];
+        }
+        int ex = block_exclusive_scan(t, &total_s) + carry;
+#pragma unroll
+        for (int j = 0; j < SC_ITEMS; ++j) {
+            if (at + j < nb) sums[at + j] = ex;
+            ex += v[j];
+        }
+        carry += total_s;
         __syncthreads();
     }
+    if (threadIdx.x == 0) sums[nb] = carry;
 }
 
 __global__ void __launch_bounds__(SC_THREADS) k_scan_down(const int *in, int *out, int64_t n,
@@ -257,110 +333,225 @@ int exclusive_scan(const int *in, int *out, int64_t n, cudaStream_t s, int64_t *
 }
 
 // ---------------------------------------------------------------------------
-// stable LSD radix sort of (uint64 key, uint32 value) pairs, 8 bits a pass
+// stable LSD radix sort of (uint64 key, value) pairs, at most 8 bits a pass.
+// A pass is three kernels: digit counts per tile, a scan of each digit's
+// counts over the tiles (one block per digit), and the scatter.  The
+// scatter is the cost: its blocks order their tile in shared memory first, so
+// that consecutive threads write runs of a digit to consecutive addresses.
+// Writing each pair from where it was read touched a sector per pair: 161 us
+// a pass on 8.4M pairs (and 49 counting, 23 scanning); now 63, 12.5 and 3.
 // ---------------------------------------------------------------------------
-constexpr int RS_THREADS = 256, RS_WARPS = RS_THREADS / 32, RS_ITEMS = 16;
-constexpr int RS_WARP_TILE = 32 * RS_ITEMS, RS_TILE = RS_THREADS * RS_ITEMS;
+constexpr int RS_BITS = 8, RS_BINS = 1 << RS_BITS;
+constexpr int RS_THREADS = 512, RS_WARPS = RS_THREADS / 32;
+// keys per thread: two scatter blocks per SM by shared memory
+template <typename W>
+constexpr int RS_ITEMS = sizeof(W) <= 4 ? 16 : 8;
+template <typename W>
+constexpr int RS_TILE = RS_THREADS * RS_ITEMS<W>;
 
-__global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const uint64_t *keys, int64_t n,
-                                                           int shift, unsigned *hist, int nblocks) {
-    __shared__ unsigned h[256];
-    for (int i = threadIdx.x; i < 256; i += RS_THREADS) h[i] = 0;
-    __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    unsigned lane = threadIdx.x & 31;
-    for (int k = threadIdx.x; k < RS_TILE; k += RS_THREADS) {
-        int64_t i = base + k;
-        bool valid = i < n;
-        unsigned d = valid ? (unsigned)((keys[i] >> shift) & 255u) : 256u;
-        unsigned peers = __match_any_sync(FULL, d);
-        if (valid && lane == (unsigned)(31 - __clz(peers))) atomicAdd(&h[d], (unsigned)__popc(peers));
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < 256; d += RS_THREADS) hist[(int64_t)d * nblocks + blockIdx.x] = h[d];
+// dynamic shared memory of the scatter: the tile's keys and values, the
+// warps' digit counts, the digits' offsets
+template <typename W>
+constexpr size_t RS_SMEM = RS_TILE<W> * (sizeof(uint64_t) + sizeof(W)) + sizeof(unsigned) * RS_BINS +
+                           sizeof(uint16_t) * RS_WARPS * RS_BINS;
+
+__device__ __forceinline__ unsigned rs_digit(uint64_t key, int shift, unsigned mask) {
+    return (unsigned)(key >> shift) & mask;
 }
 
-__global__ void __launch_bounds__(RS_THREADS) k_radix_scatter(const uint64_t *kin, const uint32_t *vin,
-                                                              uint64_t *kout, uint32_t *vout, int64_t n,
-                                                              int shift, const int *offsets, int nblocks) {
-    __shared__ unsigned wh[RS_WARPS][256];
-    __shared__ unsigned boff[256];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) (&wh[0][0])[i] = 0;
-    for (int d = threadIdx.x; d < 256; d += RS_THREADS)
-        boff[d] = (unsigned)offsets[(int64_t)d * nblocks + blockIdx.x];
-    __syncthreads();
-    const int64_t wbase = (int64_t)blockIdx.x * RS_TILE + (int64_t)warp * RS_WARP_TILE;
-    const unsigned lt = (1u << lane) - 1u;
-    unsigned loc[RS_ITEMS];
+// lanes whose digit equals this lane's (RS_BINS: no key): one ballot per bit
+// (match.any takes some 50 cycles of the SM for 32 different digits)
+__device__ __forceinline__ unsigned rs_peers(unsigned d) {
+    unsigned peers = FULL;
 #pragma unroll
-    for (int r = 0; r < RS_ITEMS; ++r) {
-        int64_t i = wbase + r * 32 + lane;
-        bool valid = i < n;
-        unsigned d = valid ? (unsigned)((kin[i] >> shift) & 255u) : 256u;
-        unsigned peers = __match_any_sync(FULL, d);
-        unsigned cnt = valid ? wh[warp][d] : 0u;
-        __syncwarp();
-        if (valid && lane == 31 - __clz(peers)) wh[warp][d] = cnt + __popc(peers);
-        __syncwarp();
-        loc[r] = cnt + __popc(peers & lt);
+    for (int b = 0; b <= RS_BITS; ++b) {
+        const unsigned set = __ballot_sync(FULL, (d >> b) & 1u);
+        peers &= (d >> b) & 1u ? set : ~set;
+    }
+    return peers;
+}
+
+// hist[d * nblocks + b]: keys of tile b with digit d
+template <int ITEMS>
+__global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const uint64_t *keys, int64_t n, int shift, unsigned mask,
+                                                           unsigned *hist, int nblocks) {
+    __shared__ unsigned h[RS_BINS];
+    for (int i = threadIdx.x; i < RS_BINS; i += RS_THREADS) h[i] = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * (RS_THREADS * ITEMS);
+    unsigned d[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int64_t i = base + r * RS_THREADS + threadIdx.x;
+        d[r] = i < n ? rs_digit(__ldg(keys + i), shift, mask) : RS_BINS;
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r)
+        if (d[r] < RS_BINS) atomicAdd(&h[d[r]], 1u);  // grouping equal digits first costs more than their conflicts
+    __syncthreads();
+    for (int d = threadIdx.x; d < RS_BINS; d += RS_THREADS) hist[(int64_t)d * nblocks + blockIdx.x] = h[d];
+}
+
+// block d: exclusive scan of digit d's counts over the tiles, and their total
+__global__ void __launch_bounds__(SC_THREADS) k_radix_scan(int *hist, int nblocks, int *totals) {
+    __shared__ int total_s;
+    int *row = hist + (int64_t)blockIdx.x * nblocks;
+    int carry = 0;
+    for (int base = 0; base < nblocks; base += SC_TILE) {
+        const int at = base + threadIdx.x * SC_ITEMS;
+        int v[SC_ITEMS], t = 0;
+#pragma unroll
+        for (int j = 0; j < SC_ITEMS; ++j) {
+            v[j] = at + j < nblocks ? row[at + j] : 0;
+            t += v[j];
+        }
+        int ex = block_exclusive_scan(t, &total_s) + carry;
+#pragma unroll
+        for (int j = 0; j < SC_ITEMS; ++j) {
+            if (at + j < nblocks) row[at + j] = ex;
+            ex += v[j];
+        }
+        carry += total_s;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
+}
+
+// exclusive scan of RS_BINS values by the block's first RS_BINS threads (the
+// whole block calls it)
+__device__ __forceinline__ unsigned scan_bins(unsigned v) {
+    __shared__ unsigned ws[RS_BINS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned incl = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned t = __shfl_up_sync(FULL, incl, d);
+        if (lane >= d) incl += t;
     }
     __syncthreads();
-    for (int d = threadIdx.x; d < 256; d += RS_THREADS) {
-        unsigned run = 0;
+    if (warp < RS_BINS / 32 && lane == 31) ws[warp] = incl;
+    __syncthreads();
+    unsigned before = 0;
+    for (int w = 0; w < RS_BINS / 32 && w < warp; ++w) before += ws[w];
+    return before + incl - v;
+}
+
+template <typename W>
+__global__ void __launch_bounds__(RS_THREADS, 2)
+k_radix_scatter(const uint64_t *__restrict__ kin, const W *__restrict__ vin, uint64_t *__restrict__ kout,
+                W *__restrict__ vout, int64_t n, int shift, unsigned mask, const int *__restrict__ offsets,
+                const int *__restrict__ totals, int nblocks) {
+    constexpr int ITEMS = RS_ITEMS<W>, TILE = RS_TILE<W>;
+    extern __shared__ __align__(16) unsigned char rs_smem[];
+    uint64_t *sk = reinterpret_cast<uint64_t *>(rs_smem);
+    W *sv = reinterpret_cast<W *>(sk + TILE);
+    unsigned *delta = reinterpret_cast<unsigned *>(sv + TILE);  // global minus local position of a digit's first pair
+    uint16_t *wh = reinterpret_cast<uint16_t *>(delta + RS_BINS);  // [warp][digit]: counts, then local positions
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int i = tid; i < RS_WARPS * RS_BINS / 2; i += RS_THREADS) reinterpret_cast<unsigned *>(wh)[i] = 0;
+    const int64_t base = (int64_t)blockIdx.x * TILE;
+    const int count = (int)(n - base < TILE ? n - base : TILE);
+    const int wbase = warp * 32 * ITEMS;
+    const unsigned lt = (1u << lane) - 1u;
+    uint16_t *mine = wh + warp * RS_BINS;
+    uint64_t k[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int i = wbase + r * 32 + lane;
+        k[r] = i < count ? kin[base + i] : 0;
+    }
+    __syncthreads();
+    unsigned loc[ITEMS / 2];  // ranks among the warp's earlier pairs of the digit (below 2^16, two a word)
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const bool valid = wbase + r * 32 + lane < count;
+        const unsigned d = valid ? rs_digit(k[r], shift, mask) : RS_BINS;
+        const unsigned peers = rs_peers(d);
+        const unsigned cnt = valid ? mine[d] : 0u;
+        __syncwarp();
+        if (valid && lane == 31 - __clz(peers)) mine[d] = (uint16_t)(cnt + __popc(peers));
+        __syncwarp();
+        const unsigned rank = cnt + __popc(peers & lt);
+        loc[r / 2] = r % 2 ? loc[r / 2] | (rank << 16) : rank;
+    }
+    __syncthreads();
+    // per digit: pairs of earlier warps, of the tile, and where the digit starts
+    unsigned run = 0;
+    if (tid < RS_BINS)
         for (int w = 0; w < RS_WARPS; ++w) {
-            unsigned c = wh[w][d];
-            wh[w][d] = run;
+            const unsigned c = wh[w * RS_BINS + tid];
+            wh[w * RS_BINS + tid] = (uint16_t)run;
             run += c;
         }
+    const unsigned local = scan_bins(tid < RS_BINS ? run : 0u);
+    const unsigned global = scan_bins(tid < RS_BINS ? (unsigned)totals[tid] : 0u);
+    if (tid < RS_BINS) {
+        for (int w = 0; w < RS_WARPS; ++w) wh[w * RS_BINS + tid] = (uint16_t)(wh[w * RS_BINS + tid] + local);
+        delta[tid] = global + (unsigned)offsets[(int64_t)tid * nblocks + blockIdx.x] - local;
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < RS_ITEMS; ++r) {
-        int64_t i = wbase + r * 32 + lane;
-        if (i < n) {
-            uint64_t k = kin[i];
-            unsigned d = (unsigned)((k >> shift) & 255u);
-            unsigned pos = boff[d] + wh[warp][d] + loc[r];
-            kout[pos] = k;
-            vout[pos] = vin[i];
+    for (int r = 0; r < ITEMS; ++r) {
+        const int i = wbase + r * 32 + lane;
+        if (i < count) {
+            const unsigned pos = mine[rs_digit(k[r], shift, mask)] + ((loc[r / 2] >> (r % 2 * 16)) & 0xffffu);
+            sk[pos] = k[r];
+            sv[pos] = vin[base + i];
         }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int i = tid; i < count; i += RS_THREADS) {
+        const uint64_t key = sk[i];
+        const unsigned at = delta[rs_digit(key, shift, mask)] + (unsigned)i;
+        kout[at] = key;
+        vout[at] = sv[i];
     }
 }
 
-// Sorts keys[0..n) with their values; the result is left in (*kres, *vres),
-// which point either at the inputs or at the scratch pair (kalt, valt).
-int radix_sort_pairs(uint64_t *keys, uint32_t *vals, uint64_t *kalt, uint32_t *valt, int64_t n,
-                     int total_bits, cudaStream_t s, uint64_t **kres, uint32_t **vres) {
-    int nblocks = (int)((n + RS_TILE - 1) / RS_TILE);
+// Sorts keys[0..n) with their values of type W, read from vin and left, as the
+// keys, in one of the two buffers of (keys, kalt) and (v0, v1).  vin may be v0.
+template <typename W>
+int radix_sort_pairs(uint64_t *keys, const W *vin, uint64_t *kalt, W *v0, W *v1, int64_t n, int total_bits,
+                     cudaStream_t s, uint64_t **kres, W **vres) {
+    const int nblocks = (int)((n + RS_TILE<W> - 1) / RS_TILE<W>);
     Tmp<int> hist;
-    SPMV_TRY(hist.alloc((size_t)256 * nblocks, s));
+    SPMV_TRY(hist.alloc((size_t)RS_BINS * nblocks + RS_BINS, s));
+    int *totals = hist.p + (size_t)RS_BINS * nblocks;
+    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)k_radix_scatter<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)RS_SMEM<W>));
     uint64_t *ka = keys, *kb = kalt;
-    uint32_t *va = vals, *vb = valt;
-    for (int shift = 0; shift < total_bits; shift += 8) {
-        k_radix_hist<<<nblocks, RS_THREADS, 0, s>>>(ka, n, shift, reinterpret_cast<unsigned *>(hist.p),
-                                                    nblocks);
-        SPMV_TRY(exclusive_scan(hist.p, hist.p, (int64_t)256 * nblocks, s, nullptr));
-        k_radix_scatter<<<nblocks, RS_THREADS, 0, s>>>(ka, va, kb, vb, n, shift, hist.p, nblocks);
+    W *vb = v1, *vo = v0;
+    // passes of nearly equal width
+    const int passes = (total_bits + RS_BITS - 1) / RS_BITS;
+    int shift = 0;
+    for (int p = 0; p < passes; ++p) {
+        const int bits = (total_bits - shift + passes - p - 1) / (passes - p);
+        const unsigned mask = (1u << bits) - 1u;
+        k_radix_hist<RS_ITEMS<W>><<<nblocks, RS_THREADS, 0, s>>>(ka, n, shift, mask,
+                                                                 reinterpret_cast<unsigned *>(hist.p), nblocks);
+        k_radix_scan<<<RS_BINS, SC_THREADS, 0, s>>>(hist.p, nblocks, totals);
+        k_radix_scatter<W><<<nblocks, RS_THREADS, RS_SMEM<W>, s>>>(ka, vin, kb, vb, n, shift, mask, hist.p, totals,
+                                                                   nblocks);
         SPMV_CUDA_TRY(cudaGetLastError());
         std::swap(ka, kb);
-        std::swap(va, vb);
+        vin = vb;
+        std::swap(vb, vo);
+        shift += bits;
     }
     *kres = ka;
-    *vres = va;
+    *vres = vo;
     return SPMV_OK;
 }
 
 // ---------------------------------------------------------------------------
 // unsorted / duplicated triplets: sort by (row, col), merge duplicates
 // ---------------------------------------------------------------------------
-__global__ void k_make_keys(const int *rows, const int *cols, int64_t nnz, int colbits,
-                            uint64_t *keys, uint32_t *idx) {
+__global__ void k_make_keys(const int *rows, const int *cols, int64_t nnz, int colbits, uint64_t *keys) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += stride) {
-        keys[i] = ((uint64_t)(uint32_t)rows[i] << colbits) | (uint32_t)cols[i];
-        idx[i] = (uint32_t)i;
-    }
+#pragma unroll 4
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += stride)
+        keys[i] = ((uint64_t)(uint32_t)__ldg(rows + i) << colbits) | (uint32_t)__ldg(cols + i);
 }
 
 __global__ void k_heads(const uint64_t *keys, int64_t n, int *head) {
@@ -376,33 +567,122 @@ __device__ __forceinline__ void from_acc(double a, double *o) { *o = a; }
 __device__ __forceinline__ void from_acc(float a, float *o) { *o = a; }
 __device__ __forceinline__ void from_acc(float a, __nv_bfloat16 *o) { *o = __float2bfloat16_rn(a); }
 
-// each run of equal keys becomes one entry; its value is the sum of the
-// run's values in original triplet order (the sort is stable)
-template <typename V, typename T>
-__global__ void k_merge_runs(const uint64_t *keys, const uint32_t *perm, const V *vin,
-                             const int *head, const int *pos, int64_t n, int colbits,
-                             int *urows, int *ucols, V *uvals) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const uint64_t mask = (uint64_t(1) << colbits) - 1;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        if (!head[i]) continue;
-        uint64_t k = keys[i];
-        T acc = to_acc(vin[perm[i]]);
-        for (int64_t j = i + 1; j < n && !head[j]; ++j) acc += to_acc(vin[perm[j]]);
-        int u = pos[i];
-        urows[u] = (int)(k >> colbits);
-        ucols[u] = (int)(k & mask);
-        from_acc(acc, &uvals[u]);
+// Each run of equal keys becomes one entry; its value is the sum of the run's
+// values in original triplet order (the sort is stable).  Two passes over the
+// keys: heads per tile, then (after a scan of the tiles) the entries
+// themselves; no head or position array is written.  A warp takes 256
+// consecutive keys, 32 a step, so that loads and the stores of the entries
+// (mostly one per key) are contiguous (eight keys in a row per thread: 160 us
+// on 8.4M triplets, bound by partial-sector writes; 50 now,
+// and 11 counting, against 156 with head and position arrays and a gather of
+// the values through a sorted index).
+__device__ __forceinline__ void head_masks(const uint64_t *__restrict__ keys, int64_t w0, int64_t n,
+                                           uint64_t (&k)[SC_ITEMS], unsigned (&mask)[SC_ITEMS]) {
+    const int lane = threadIdx.x & 31;
+    uint64_t prev = lane == 0 && w0 > 0 && w0 < n ? __ldg(keys + w0 - 1) : 0;  // of lane 0: the key before the step
+#pragma unroll
+    for (int j = 0; j < SC_ITEMS; ++j) k[j] = w0 + 32 * j + lane < n ? __ldg(keys + w0 + 32 * j + lane) : 0;
+#pragma unroll
+    for (int j = 0; j < SC_ITEMS; ++j) {
+        const int64_t i = w0 + 32 * j + lane;
+        const uint64_t up = __shfl_up_sync(FULL, k[j], 1), last = __shfl_sync(FULL, k[j], 31);
+        const uint64_t before = lane == 0 ? prev : up;
+        mask[j] = __ballot_sync(FULL, i < n && (i == 0 || k[j] != before));
+        prev = last;
     }
 }
 
+__global__ void __launch_bounds__(SC_THREADS) k_merge_count(const uint64_t *keys, int64_t n, int *sums) {
+    __shared__ int ws[SC_THREADS / 32];
+    const int warp = threadIdx.x >> 5;
+    uint64_t k[SC_ITEMS];
+    unsigned mask[SC_ITEMS];
+    head_masks(keys, (int64_t)blockIdx.x * SC_TILE + 32 * SC_ITEMS * warp, n, k, mask);
+    int c = 0;
+#pragma unroll
+    for (int j = 0; j < SC_ITEMS; ++j) c += __popc(mask[j]);
+    if ((threadIdx.x & 31) == 0) ws[warp] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int w = 0; w < SC_THREADS / 32; ++w) t += ws[w];
+        sums[blockIdx.x] = t;
+    }
+}
+
+template <typename V, typename T>
+__global__ void __launch_bounds__(SC_THREADS)
+k_merge_runs(const uint64_t *__restrict__ keys, const V *__restrict__ vin, const int *__restrict__ sums, int64_t n, int colbits, int *urows, int *ucols, V *uvals) {
+    __shared__ int ws[SC_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t w0 = (int64_t)blockIdx.x * SC_TILE + 32 * SC_ITEMS * warp;
+    const uint64_t colmask = (uint64_t(1) << colbits) - 1;
+    uint64_t k[SC_ITEMS];
+    unsigned mask[SC_ITEMS];
+    head_masks(keys, w0, n, k, mask);
+    T v[SC_ITEMS];
+    int c = 0;
+#pragma unroll
+    for (int j = 0; j < SC_ITEMS; ++j) {
+        c += __popc(mask[j]);
+        if ((mask[j] >> lane) & 1u) v[j] = to_acc(vin[w0 + 32 * j + lane]);
+    }
+    if (lane == 0) ws[warp] = c;
+    __syncthreads();
+    int u0 = sums[blockIdx.x];
+    for (int w = 0; w < warp; ++w) u0 += ws[w];
+#pragma unroll
+    for (int j = 0; j < SC_ITEMS; ++j) {
+        if ((mask[j] >> lane) & 1u) {
+            T acc = v[j];
+            for (int64_t i = w0 + 32 * j + lane + 1; i < n && keys[i] == k[j]; ++i) acc += to_acc(vin[i]);
+            const int u = u0 + __popc(mask[j] & ((1u << lane) - 1u));
+            urows[u] = (int)(k[j] >> colbits);
+            ucols[u] = (int)(k[j] & colmask);
+            from_acc(acc, &uvals[u]);
+        }
+        u0 += __popc(mask[j]);
+    }
+}
+
+// The unordered path of build_csr: triplets sorted by (row, col) with their
+// values as the sort's payload (a gather through a sorted index cost more than
+// the values' way through the passes), then merged.  Sets h->nnz, h->colidx,
+// h->vals and the row of every entry in `urows`.
 template <typename V>
-int merge_dispatch(const uint64_t *keys, const uint32_t *perm, const void *vin, const int *head,
-                   const int *pos, int64_t n, int colbits, int *urows, int *ucols, void *uvals,
-                   cudaStream_t s) {
+int sort_and_merge(spmv_matrix *h, const int32_t *d_rows, const int32_t *d_cols, const void *d_vals, int64_t nnz,
+                   cudaStream_t s, Tmp<int> *urows) {
     using T = typename std::conditional<std::is_same<V, double>::value, double, float>::type;
-    k_merge_runs<V, T><<<grid1d(n, 256), 256, 0, s>>>(keys, perm, (const V *)vin, head, pos, n, colbits,
-                                                       urows, ucols, (V *)uvals);
+    using W = typename std::conditional<sizeof(V) == 8, uint64_t,
+                                        typename std::conditional<sizeof(V) == 4, uint32_t, uint16_t>::type>::type;
+    const int colbits = std::max(1, bits_for(h->n));
+    Tmp<uint64_t> k0, k1;
+    Tmp<W> v0, v1;
+    SPMV_TRY(k0.alloc(nnz, s));
+    SPMV_TRY(k1.alloc(nnz, s));
+    SPMV_TRY(v0.alloc(nnz, s));
+    SPMV_TRY(v1.alloc(nnz, s));
+    k_make_keys<<<grid1d(nnz, 256, 152 * 16), 256, 0, s>>>(d_rows, d_cols, nnz, colbits, k0.p);
+    uint64_t *ks;
+    W *vsorted;
+    SPMV_TRY(radix_sort_pairs<W>(k0.p, static_cast<const W *>(d_vals), k1.p, v0.p, v1.p, nnz, bits_for(h->m) + colbits,
+                                 s, &ks, &vsorted));
+    const int64_t nb = (nnz + SC_TILE - 1) / SC_TILE;
+    Tmp<int> sums;
+    SPMV_TRY(sums.alloc(nb + 1, s));
+    k_merge_count<<<(unsigned)nb, SC_THREADS, 0, s>>>(ks, nnz, sums.p);
+    k_scan_sums<<<1, SC_THREADS, 0, s>>>(sums.p, nb);
+    SPMV_CUDA_TRY(cudaGetLastError());
+    int nu = 0;
+    SPMV_CUDA_TRY(cudaMemcpyAsync(&nu, sums.p + nb, sizeof(int), cudaMemcpyDeviceToHost, s));
+    SPMV_CUDA_TRY(cudaStreamSynchronize(s));
+    h->nnz = nu;
+    SPMV_TRY(urows->alloc(nu, s));
+    SPMV_TRY(dalloc(&h->colidx, (size_t)nu + CSR_PAD));
+    SPMV_TRY(dalloc_bytes(&h->vals, sizeof(V) * (nu + CSR_PAD)));
+    k_merge_runs<V, T><<<(unsigned)nb, SC_THREADS, 0, s>>>(ks, reinterpret_cast<const V *>(vsorted), sums.p, nnz, colbits,
+                                                           urows->p, h->colidx, (V *)h->vals);
+    SPMV_CUDA_TRY(cudaGetLastError());
     return SPMV_OK;
 }
 
@@ -416,20 +696,52 @@ __device__ __forceinline__ void ell_code(int16_t *p, int c, int64_t r) {
     *p = c < 0 ? (int16_t)INT16_MIN : (int16_t)(c - r);
 }
 
+// A warp packs 32 rows.  Their entries are contiguous in CSR: they are staged
+// in shared memory with contiguous loads (at most `cap` entries; longer ranges
+// are read in place, a row per lane) and leave column by column, 32 slots a
+// store.  Reading a row per lane touched 32 lines a load: 27-point stencil
+// 101^3, fp64, 216 us, 156 now (its bytes at the HBM rate: 98), bound by
+// load latency at the 20 warps per SM that the staging leaves room for.
+// One padding word per 32 spreads rows of one length over the banks.
+constexpr int ELL_PACK_CAP = 4608, ELL_PACK_SMEM = 96 * 1024;
+__host__ __device__ inline size_t ell_pack_words(int cap) { return (size_t)cap + cap / 32 + 1; }
+
 template <typename V, typename CI>
-__global__ void k_ell_pack(const int *rowptr, const int *colidx, const V *vals, int64_t m,
-                           int64_t width, int64_t pitch, CI *ell_col, V *ell_val) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < pitch; r += stride) {
-        int64_t s = 0, len = 0;
-        if (r < m) {
-            s = rowptr[r];
-            len = rowptr[r + 1] - s;
+__global__ void __launch_bounds__(128) k_ell_pack(const int *__restrict__ rowptr, const int *__restrict__ colidx,
+                                                  const V *__restrict__ vals, int64_t m, int64_t width, int64_t pitch,
+                                                  int cap, CI *ell_col, V *ell_val) {
+    extern __shared__ __align__(16) unsigned char pack_smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const size_t words = ell_pack_words(cap);
+    V *sv = reinterpret_cast<V *>(pack_smem) + warp * words;
+    int *sc = reinterpret_cast<int *>(pack_smem + (sizeof(V) * words * nw + 15) / 16 * 16) + warp * words;
+    const int64_t stride = (int64_t)gridDim.x * nw * 32;
+    for (int64_t base = ((int64_t)blockIdx.x * nw + warp) * 32; base < pitch; base += stride) {
+        const int64_t r = base + lane;
+        const int s = __ldg(rowptr + (r < m ? r : m)), e = __ldg(rowptr + (r + 1 < m ? r + 1 : m));
+        const int w0 = __shfl_sync(FULL, s, 0), w1 = __shfl_sync(FULL, e, 31);
+        const bool staged = w1 - w0 <= cap;
+        __syncwarp();
+        if (staged) {
+#pragma unroll 8
+            for (int o = lane; o < w1 - w0; o += 32) {
+                sc[o + (o >> 5)] = __ldg(colidx + w0 + o);
+                sv[o + (o >> 5)] = vals[w0 + o];
+            }
         }
-        for (int64_t k = 0; k < width; ++k) {
-            bool have = k < len;
-            ell_code(ell_col + k * pitch + r, have ? colidx[s + k] : -1, r);
-            ell_val[k * pitch + r] = have ? vals[s + k] : V(0.0f);
+        __syncwarp();
+        const int len = e - s, first = s - w0;
+#pragma unroll 4
+        for (int k = 0; k < (int)width; ++k) {
+            int c = -1;
+            V v = V(0.0f);
+            if (k < len) {
+                const int o = first + k;
+                c = staged ? sc[o + (o >> 5)] : __ldg(colidx + s + k);
+                v = staged ? sv[o + (o >> 5)] : vals[s + k];
+            }
+            ell_code(ell_col + k * pitch + r, c, r);
+            ell_val[k * pitch + r] = v;
         }
     }
 }
@@ -594,11 +906,11 @@ __global__ void k_long_fill(const int *rowptr, int64_t nrows, int64_t threshold,
 
 // SELL: sort key per row = descending length (the sort is stable, so rows of
 // equal length keep their order)
-__global__ void k_sell_keys(const int *rowptr, int64_t m, uint64_t *keys, uint32_t *idx) {
+__global__ void k_sell_keys(const int *rowptr, int64_t m, int longest, uint64_t *keys, uint32_t *idx) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m; r += stride) {
         const int len = rowptr[r + 1] - rowptr[r];
-        keys[r] = (uint64_t)(uint32_t)(0x7fffffff - len);
+        keys[r] = (uint64_t)(uint32_t)(longest - len);
         idx[r] = (uint32_t)r;
     }
 }
@@ -622,34 +934,37 @@ __host__ __device__ __forceinline__ int64_t sell_slot(int64_t base, int64_t w, i
     return k < w4 ? base + 128 * (k >> 2) + 4 * l + (k & 3) : base + 32 * w4 + 32 * (k - w4) + l;
 }
 
-// one warp per entry index k of a slice (slices hold 32 slots per column,
-// so the warp finds (sl, k) from its 32-slot index with one binary search,
-// the same address in every lane) and lane l fills sorted row 32 sl + l
+// A warp fills a work item (at most kmax columns of a slice): lane l walks its
+// row's entries in order, so that its loads stay in one line for a while, and
+// the stores of a column are contiguous.  (A warp per column found its slice
+// by a binary search for every 32 slots.)
 template <typename V>
-__global__ void k_sell_fill(const int *rowptr, const int *colidx, const V *vals, const uint32_t *perm, int64_t m,
-                            int64_t nslices, const int *sptr, int64_t total, int *scol, V *sval, int *sperm,
-                            bool grouped) {
+__global__ void k_sell_fill(const int *__restrict__ rowptr, const int *__restrict__ colidx, const V *__restrict__ vals,
+                            const uint32_t *__restrict__ perm, int64_t m, const int *__restrict__ sptr, int64_t nitems,
+                            const int *__restrict__ it_slice, const int *__restrict__ it_base,
+                            const int *__restrict__ it_len, int *scol, V *sval, int *sperm, bool grouped) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t w = warp; w < total / 32; w += nwarps) {
-        const int64_t p0 = 32 * w;
-        const int sl = row_of(sptr, nslices, p0);
-        const int64_t k = (p0 - sptr[sl]) / 32;
+    for (int64_t it = warp; it < nitems; it += nwarps) {
+        const int sl = __ldg(it_slice + it), len = __ldg(it_len + it);
+        const int sbase = __ldg(sptr + sl), w = (__ldg(sptr + sl + 1) - sbase) / 32, k0 = (__ldg(it_base + it) - sbase) / 32;
         const int64_t q = (int64_t)sl * 32 + lane;
-        int c = -1;
-        V v = V(0.0f);
+        int rs = 0, n = 0;  // the lane's row
         if (q < m) {
-            const uint32_t r = perm[q];
-            const int64_t rs = rowptr[r];
-            if (k < rowptr[r + 1] - rs) {
-                c = colidx[rs + k];
-                v = vals[rs + k];
-            }
+            const uint32_t r = __ldg(perm + q);
+            rs = __ldg(rowptr + r);
+            n = __ldg(rowptr + r + 1) - rs;
         }
-        const int64_t at = sell_slot(sptr[sl], (sptr[sl + 1] - sptr[sl]) / 32, k, lane, grouped);
-        scol[at] = c;
-        sval[at] = v;
+#pragma unroll 4
+        for (int k = k0; k < k0 + len; ++k) {
+            const bool have = k < n;
+            const int c = have ? __ldg(colidx + rs + k) : -1;
+            const V v = have ? vals[rs + k] : V(0.0f);
+            const int64_t at = sell_slot(sbase, w, k, lane, grouped);
+            scol[at] = c;
+            sval[at] = v;
+        }
     }
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < m; q += stride) sperm[q] = (int)perm[q];
@@ -814,7 +1129,8 @@ int check_triplet_bounds(const int32_t *d_rows, const int32_t *d_cols, int64_t n
     Tmp<unsigned> flags;
     SPMV_TRY(flags.alloc(1, s));
     SPMV_CUDA_TRY(cudaMemsetAsync(flags.p, 0, sizeof(unsigned), s));
-    k_check_triplets<<<grid1d(nnz, 256), 256, 0, s>>>(d_rows, d_cols, nnz, m, n, flags.p);
+    k_check_triplets<<<grid1d(nnz, 256 * CHECK_STEPS, 152 * 8), 256, 0, s>>>(d_rows, d_cols, nnz, m, n, flags.p, nullptr,
+                                                                         nullptr);
     SPMV_CUDA_TRY(cudaGetLastError());
     unsigned hflags = 0;
     SPMV_CUDA_TRY(cudaMemcpyAsync(&hflags, flags.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
@@ -910,12 +1226,6 @@ int gather_panel(const int32_t *d_rows, const int32_t *d_cols, const void *d_val
     return SPMV_OK;
 }
 
-// The CSR arrays are allocated CSR_PAD entries longer than needed: the
-// staged tile kernel copies whole multiples of 8 column/value entries and
-// 16-byte windows of row pointers, so the last tile may read up to 7 entries
-// past nnz and 3 past m (never used).
-constexpr size_t CSR_PAD = 8;
-
 int build_csr(spmv_matrix *h, const int32_t *d_rows, const int32_t *d_cols, const void *d_vals,
               cudaStream_t s) {
     const int64_t m = h->m, n = h->n, nnz_in = h->nnz;
@@ -929,14 +1239,26 @@ int build_csr(spmv_matrix *h, const int32_t *d_rows, const int32_t *d_cols, cons
         SPMV_CUDA_TRY(cudaStreamSynchronize(s));
         return SPMV_OK;
     }
-    Tmp<unsigned> flags;
-    SPMV_TRY(flags.alloc(1, s));
-    SPMV_CUDA_TRY(cudaMemsetAsync(flags.p, 0, sizeof(unsigned), s));
-    k_check_triplets<<<grid1d(nnz_in, 256), 256, 0, s>>>(d_rows, d_cols, nnz_in, m, n, flags.p);
-    SPMV_CUDA_TRY(cudaGetLastError());
-    unsigned hflags = 0;
-    SPMV_CUDA_TRY(cudaMemcpyAsync(&hflags, flags.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-    SPMV_CUDA_TRY(cudaStreamSynchronize(s));
+    // [0] flags, [1] longest row, [2] contiguous pairs, [3] longest rows of 32-row groups; for an
+    // ordered list the first look at the triplets gives them all
+    Tmp<unsigned long long> st;
+    SPMV_TRY(st.alloc(4, s));
+    unsigned long long hst[4] = {0, 0, 0, 0};
+    auto row_statistics = [&]() {
+        k_max_row<<<grid1d(m, 1024, 152), 1024, 0, s>>>(h->rowptr, m, st.p + 1, st.p + 3);
+    };
+    auto read_statistics = [&]() -> int {
+        SPMV_CUDA_TRY(cudaGetLastError());
+        SPMV_CUDA_TRY(cudaMemcpyAsync(hst, st.p, sizeof(hst), cudaMemcpyDeviceToHost, s));
+        SPMV_CUDA_TRY(cudaStreamSynchronize(s));
+        return SPMV_OK;
+    };
+    SPMV_CUDA_TRY(cudaMemsetAsync(st.p, 0, sizeof(hst), s));
+    k_check_triplets<<<grid1d(nnz_in, 256 * CHECK_STEPS, 152 * 8), 256, 0, s>>>(
+        d_rows, d_cols, nnz_in, m, n, reinterpret_cast<unsigned *>(st.p), h->rowptr, st.p + 2);
+    row_statistics();
+    SPMV_TRY(read_statistics());
+    const unsigned hflags = (unsigned)hst[0];
     if (hflags & 1u) {
         set_error("spmv_create: a triplet lies outside the %lld x %lld matrix", (long long)m,
                   (long long)n);
@@ -949,53 +1271,28 @@ int build_csr(spmv_matrix *h, const int32_t *d_rows, const int32_t *d_cols, cons
         SPMV_TRY(dalloc_bytes(&h->vals, vs * (nnz_in + CSR_PAD)));
         SPMV_CUDA_TRY(cudaMemcpyAsync(h->colidx, d_cols, sizeof(int) * nnz_in, cudaMemcpyDeviceToDevice, s));
         SPMV_CUDA_TRY(cudaMemcpyAsync(h->vals, d_vals, vs * nnz_in, cudaMemcpyDeviceToDevice, s));
-        k_rowptr_from_sorted<<<grid1d(m + 1, 256), 256, 0, s>>>(d_rows, nnz_in, m, h->rowptr);
-        SPMV_CUDA_TRY(cudaGetLastError());
+        if (hflags & 8u) {  // long runs of empty rows: every row pointer by a search
+            SPMV_CUDA_TRY(cudaMemsetAsync(st.p + 1, 0, sizeof(unsigned long long), s));
+            SPMV_CUDA_TRY(cudaMemsetAsync(st.p + 3, 0, sizeof(unsigned long long), s));
+            k_rowptr_from_sorted<<<grid1d(m + 1, 256), 256, 0, s>>>(d_rows, nnz_in, m, h->rowptr);
+            row_statistics();
+            SPMV_TRY(read_statistics());
+        }
     } else {
-        const int colbits = std::max(1, bits_for(n));
-        const int total_bits = bits_for(m) + colbits;
-        Tmp<uint64_t> k0, k1;
-        Tmp<uint32_t> v0, v1;
-        SPMV_TRY(k0.alloc(nnz_in, s));
-        SPMV_TRY(k1.alloc(nnz_in, s));
-        SPMV_TRY(v0.alloc(nnz_in, s));
-        SPMV_TRY(v1.alloc(nnz_in, s));
-        k_make_keys<<<grid1d(nnz_in, 256), 256, 0, s>>>(d_rows, d_cols, nnz_in, colbits, k0.p, v0.p);
-        uint64_t *ks;
-        uint32_t *vp;
-        SPMV_TRY(radix_sort_pairs(k0.p, v0.p, k1.p, v1.p, nnz_in, total_bits, s, &ks, &vp));
-        Tmp<int> head, pos, urows;
-        SPMV_TRY(head.alloc(nnz_in, s));
-        SPMV_TRY(pos.alloc(nnz_in, s));
-        k_heads<<<grid1d(nnz_in, 256), 256, 0, s>>>(ks, nnz_in, head.p);
-        int64_t nu = 0;
-        SPMV_TRY(exclusive_scan(head.p, pos.p, nnz_in, s, &nu));
-        h->nnz = nu;
-        SPMV_TRY(urows.alloc(nu, s));
-        SPMV_TRY(dalloc(&h->colidx, (size_t)nu + CSR_PAD));
-        SPMV_TRY(dalloc_bytes(&h->vals, vs * (nu + CSR_PAD)));
-        if (h->vt == SPMV_F64)
-            merge_dispatch<double>(ks, vp, d_vals, head.p, pos.p, nnz_in, colbits, urows.p, h->colidx, h->vals, s);
-        else if (h->vt == SPMV_F32)
-            merge_dispatch<float>(ks, vp, d_vals, head.p, pos.p, nnz_in, colbits, urows.p, h->colidx, h->vals, s);
-        else
-            merge_dispatch<__nv_bfloat16>(ks, vp, d_vals, head.p, pos.p, nnz_in, colbits, urows.p, h->colidx,
-                                          h->vals, s);
+        Tmp<int> urows;
+        if (h->vt == SPMV_F64) SPMV_TRY(sort_and_merge<double>(h, d_rows, d_cols, d_vals, nnz_in, s, &urows));
+        else if (h->vt == SPMV_F32) SPMV_TRY(sort_and_merge<float>(h, d_rows, d_cols, d_vals, nnz_in, s, &urows));
+        else SPMV_TRY(sort_and_merge<__nv_bfloat16>(h, d_rows, d_cols, d_vals, nnz_in, s, &urows));
+        const int64_t nu = h->nnz;
         k_rowptr_from_sorted<<<grid1d(m + 1, 256), 256, 0, s>>>(urows.p, nu, m, h->rowptr);
-        SPMV_CUDA_TRY(cudaGetLastError());
+        SPMV_CUDA_TRY(cudaMemsetAsync(st.p, 0, sizeof(hst), s));
+        row_statistics();
+        if (nu > 1) k_contiguous_pairs<<<grid1d(nu, 256, 152 * 8), 256, 0, s>>>(h->colidx, nu, st.p + 2);
+        SPMV_TRY(read_statistics());
     }
-    Tmp<unsigned long long> mx;   // [0]: longest row, [1]: contiguous pairs, [2]: longest rows of 32-row groups
-    SPMV_TRY(mx.alloc(3, s));
-    SPMV_CUDA_TRY(cudaMemsetAsync(mx.p, 0, 3 * sizeof(unsigned long long), s));
-    if (m > 0) k_max_row<<<grid1d(m, 256), 256, 0, s>>>(h->rowptr, m, reinterpret_cast<int *>(mx.p), mx.p + 2);
-    if (h->nnz > 1) k_contiguous_pairs<<<grid1d(h->nnz, 256), 256, 0, s>>>(h->colidx, h->nnz, mx.p + 1);
-    SPMV_CUDA_TRY(cudaGetLastError());
-    unsigned long long hmx[3] = {0, 0, 0};
-    SPMV_CUDA_TRY(cudaMemcpyAsync(hmx, mx.p, sizeof(hmx), cudaMemcpyDeviceToHost, s));
-    SPMV_CUDA_TRY(cudaStreamSynchronize(s));
-    h->max_row = (int64_t)(hmx[0] & 0xffffffffull);
-    h->group_max = m > 0 ? (double)hmx[2] / (double)((m + 31) / 32) : 0.0;
-    h->contig = h->nnz > 1 ? (double)hmx[1] / (double)(h->nnz - 1) : 0.0;
+    h->max_row = (int64_t)hst[1];
+    h->group_max = (double)hst[3] / (double)((m + 31) / 32);
+    h->contig = h->nnz > 1 ? (double)hst[2] / (double)(h->nnz - 1) : 0.0;
     return SPMV_OK;
 }
 
@@ -1030,12 +1327,12 @@ static void free_long_rows(spmv_matrix *h) {
     L = LongRows{};
 }
 
-int build_long_rows(spmv_matrix *h, const int32_t *rowptr, int64_t nrows, int64_t threshold, int64_t seg,
-                    int stride, cudaStream_t s) {
+int build_long_rows(spmv_matrix *h, const int32_t *rowptr, int64_t nrows, int64_t longest, int64_t threshold,
+                    int64_t seg, int stride, cudaStream_t s) {
     free_long_rows(h);
     LongRows &L = h->lng;
     L.threshold = threshold;
-    if (nrows == 0) return SPMV_OK;
+    if (nrows == 0 || longest <= threshold) return SPMV_OK;
     Tmp<int> cnt, off;
     SPMV_TRY(cnt.alloc(nrows, s));
     SPMV_TRY(off.alloc(nrows, s));
@@ -1087,21 +1384,25 @@ void free_packed(spmv_matrix *h) {
 
 namespace {
 
-template <typename CI>
-int launch_ell_pack(spmv_matrix *h, int64_t width, int64_t pitch, CI *cols, cudaStream_t s) {
-    const unsigned g = grid1d(pitch, 256);
-    const int64_t m = h->m;
-    if (h->vt == SPMV_F64)
-        k_ell_pack<double, CI><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const double *)h->vals, m, width, pitch,
-                                                 cols, (double *)h->ell_val);
-    else if (h->vt == SPMV_F32)
-        k_ell_pack<float, CI><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const float *)h->vals, m, width, pitch,
-                                                cols, (float *)h->ell_val);
-    else
-        k_ell_pack<__nv_bfloat16, CI><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const __nv_bfloat16 *)h->vals, m,
-                                                        width, pitch, cols, (__nv_bfloat16 *)h->ell_val);
+template <typename V, typename CI>
+int launch_ell_pack_t(spmv_matrix *h, int64_t width, int64_t pitch, CI *cols, cudaStream_t s) {
+    auto kern = k_ell_pack<V, CI>;
+    const int cap = (int)std::min<int64_t>(ELL_PACK_CAP, 32 * width);
+    const size_t per_warp = ell_pack_words(cap) * (sizeof(V) + 4);
+    const int nw = (int)std::max<size_t>(1, std::min<size_t>(4, ELL_PACK_SMEM / per_warp));
+    const size_t smem = (sizeof(V) * ell_pack_words(cap) * nw + 15) / 16 * 16 + 4 * ell_pack_words(cap) * nw;
+    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<grid1d(pitch, 32 * nw, 1 << 20), 32 * nw, smem, s>>>(h->rowptr, h->colidx, (const V *)h->vals, h->m, width,
+                                                                pitch, cap, cols, (V *)h->ell_val);
     SPMV_CUDA_TRY(cudaGetLastError());
     return SPMV_OK;
+}
+
+template <typename CI>
+int launch_ell_pack(spmv_matrix *h, int64_t width, int64_t pitch, CI *cols, cudaStream_t s) {
+    if (h->vt == SPMV_F64) return launch_ell_pack_t<double, CI>(h, width, pitch, cols, s);
+    if (h->vt == SPMV_F32) return launch_ell_pack_t<float, CI>(h, width, pitch, cols, s);
+    return launch_ell_pack_t<__nv_bfloat16, CI>(h, width, pitch, cols, s);
 }
 
 // bf16 values: columns are stored as 16-bit offsets from the row when
@@ -1224,7 +1525,7 @@ int pack_bsr(spmv_matrix *h, int r, cudaStream_t s) {
     k_block_keys<<<grid1d(nnz, 256), 256, 0, s>>>(rows.p, h->colidx, nnz, r, bcbits, k0.p, v0.p);
     uint64_t *ks;
     uint32_t *vp;
-    SPMV_TRY(radix_sort_pairs(k0.p, v0.p, k1.p, v1.p, nnz, total_bits, s, &ks, &vp));
+    SPMV_TRY(radix_sort_pairs<uint32_t>(k0.p, v0.p, k1.p, v0.p, v1.p, nnz, total_bits, s, &ks, &vp));
     Tmp<int> head, pos;
     SPMV_TRY(head.alloc(nnz, s));
     SPMV_TRY(pos.alloc(nnz, s));
@@ -1286,10 +1587,10 @@ int pack_sell(spmv_matrix *h, int kmax, bool grouped, cudaStream_t s) {
     SPMV_TRY(k1.alloc(m, s));
     SPMV_TRY(v0.alloc(m, s));
     SPMV_TRY(v1.alloc(m, s));
-    k_sell_keys<<<grid1d(m, 256), 256, 0, s>>>(h->rowptr, m, k0.p, v0.p);
+    k_sell_keys<<<grid1d(m, 256), 256, 0, s>>>(h->rowptr, m, (int)h->max_row, k0.p, v0.p);
     uint64_t *ks;
     uint32_t *perm;
-    SPMV_TRY(radix_sort_pairs(k0.p, v0.p, k1.p, v1.p, m, 32, s, &ks, &perm));
+    SPMV_TRY(radix_sort_pairs<uint32_t>(k0.p, v0.p, k1.p, v0.p, v1.p, m, std::max(1, bits_for(h->max_row + 1)), s, &ks, &perm));
     Tmp<int> slots;
     SPMV_TRY(slots.alloc(nslices + 1, s));
     SPMV_CUDA_TRY(cudaMemsetAsync(slots.p, 0, sizeof(int) * (nslices + 1), s));
@@ -1303,21 +1604,7 @@ int pack_sell(spmv_matrix *h, int kmax, bool grouped, cudaStream_t s) {
     h->sell_slots = total;
     SPMV_TRY(dalloc(&h->sell_col, (size_t)total));
     SPMV_TRY(dalloc_bytes(&h->sell_val, vs * total));
-    const unsigned g = grid1d(std::max<int64_t>(total, m), 256);
-    if (h->vt == SPMV_F64)
-        k_sell_fill<double><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const double *)h->vals, perm, m, nslices,
-                                              h->sell_ptr, total, h->sell_col, (double *)h->sell_val, h->sell_perm,
-                                              grouped);
-    else if (h->vt == SPMV_F32)
-        k_sell_fill<float><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const float *)h->vals, perm, m, nslices,
-                                             h->sell_ptr, total, h->sell_col, (float *)h->sell_val, h->sell_perm,
-                                             grouped);
-    else
-        k_sell_fill<__nv_bfloat16><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const __nv_bfloat16 *)h->vals, perm, m,
-                                                     nslices, h->sell_ptr, total, h->sell_col,
-                                                     (__nv_bfloat16 *)h->sell_val, h->sell_perm, grouped);
-    SPMV_CUDA_TRY(cudaGetLastError());
-    // work items (slice, first slot, column count <= 256) and the partials
+    // work items (slice, first slot, column count <= kmax) and the partials
     // joining the items of one slice
     LongRows &L = h->lng;
     Tmp<int> cnt, off;
@@ -1335,6 +1622,16 @@ int pack_sell(spmv_matrix *h, int kmax, bool grouped, cudaStream_t s) {
     SPMV_TRY(dalloc(&L.seg_c1, (size_t)nitems));
     k_sell_item_fill<<<grid1d(nslices, 256), 256, 0, s>>>(h->sell_ptr, nslices, kmax, off.p, L.seg_row,
                                                            L.seg_begin, L.seg_end, L.seg_c0, L.seg_c1);
+    SPMV_CUDA_TRY(cudaGetLastError());
+    const unsigned g = grid1d(std::max<int64_t>(32 * nitems, m), 256, 152 * 16);
+    auto fill = [&](auto *v) {
+        using V = std::remove_pointer_t<decltype(v)>;
+        k_sell_fill<V><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const V *)h->vals, perm, m, h->sell_ptr, nitems, L.seg_row,
+                                         L.seg_begin, L.seg_end, h->sell_col, (V *)h->sell_val, h->sell_perm, grouped);
+    };
+    if (h->vt == SPMV_F64) fill((double *)nullptr);
+    else if (h->vt == SPMV_F32) fill((float *)nullptr);
+    else fill((__nv_bfloat16 *)nullptr);
     SPMV_CUDA_TRY(cudaGetLastError());
     SPMV_TRY(alloc_partials(&L.part, nitems, 32, h->vt, s));
     // rows of the zero-width slices are written by a grid-stride pass
@@ -1427,7 +1724,7 @@ int pack_format(spmv_matrix *h, const spmv_config &cfg, cudaStream_t s) {
             const bool uneven = csr_uneven(h, cfg.threads_per_row);
             const int64_t thr =
                 uneven ? CSR_WARP_ROW : std::max<int64_t>(512, 32LL * cfg.threads_per_row * cfg.unroll);
-            SPMV_TRY(build_long_rows(h, h->rowptr, h->m, thr, uneven ? CSR_SEG_LEN : 4096, 1, s));
+            SPMV_TRY(build_long_rows(h, h->rowptr, h->m, h->max_row, thr, uneven ? CSR_SEG_LEN : 4096, 1, s));
         }
         break;
     case SPMV_FMT_ELL: {
@@ -1461,7 +1758,8 @@ int pack_format(spmv_matrix *h, const spmv_config &cfg, cudaStream_t s) {
     case SPMV_FMT_BSR: {
         SPMV_TRY(pack_bsr(h, cfg.bsr_block, s));
         const int64_t thr = 256LL * cfg.threads_per_row;
-        SPMV_TRY(build_long_rows(h, h->bsr_rowptr, h->bsr_mb, thr, 16LL * (256 / cfg.bsr_block), cfg.bsr_block, s));
+        // a block row holds at most the entries of its rows
+        SPMV_TRY(build_long_rows(h, h->bsr_rowptr, h->bsr_mb, cfg.bsr_block * h->max_row, thr, 16LL * (256 / cfg.bsr_block), cfg.bsr_block, s));
         break;
     }
     default:

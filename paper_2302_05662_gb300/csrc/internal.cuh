@@ -374,8 +374,9 @@ int build_coo_meta(const int32_t *rows, const int32_t *rowptr, int64_t nnz, int 
 int build_merge_meta(const int32_t *rowptr, int64_t m, int64_t nnz, int C, int32_t *meta, cudaStream_t s);
 int alloc_partials(Partials *p, int64_t units, int stride, int vt, cudaStream_t s);
 void free_partials(Partials *p);
-int build_long_rows(spmv_matrix *h, const int32_t *rowptr, int64_t nrows, int64_t threshold, int64_t seg,
-                    int stride, cudaStream_t s);
+// longest: an upper bound of the row lengths
+int build_long_rows(spmv_matrix *h, const int32_t *rowptr, int64_t nrows, int64_t longest, int64_t threshold,
+                    int64_t seg, int stride, cudaStream_t s);
 
 // row panels (convert.cu): bounds check of every triplet; panel row bounds
 // (multiples of 4 rows, at most `limit` triplets each); stable copy of the
