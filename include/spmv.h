@@ -83,7 +83,10 @@ typedef enum { SPMV_F64 = 0, SPMV_F32 = 1, SPMV_BF16 = 2 } spmv_dtype;
 
 typedef enum {
     SPMV_FMT_CSR = 0, /* Section 2.3: Data, Column Index, Row Index        */
-    SPMV_FMT_ELL = 1, /* Section 2.3: m x max_nnz padded, column-major     */
+    SPMV_FMT_ELL = 1, /* Section 2.3: m x max_nnz padded, column-major; large */
+                      /* matrices whose neighbouring rows share their column */
+                      /* offsets (stencils, bands) are held by diagonals of  */
+                      /* row slices, one offset instead of a column per row  */
     SPMV_FMT_COO = 2, /* (row, col, val) triplets sorted by row            */
     SPMV_FMT_HYB = 3, /* ELL part + COO overflow                           */
     SPMV_FMT_BSR = 4, /* r x r dense blocks (blocked format of Sec. 2.3)   */
@@ -106,7 +109,9 @@ typedef enum {
  * Kernel and launch parameters (Section 4, items 1-3, plus the format of
  * item 4).  A zero field takes the library default.
  *   format            spmv_format.
- *   threads_per_block 32..1024, a power of two (default 256).
+ *   threads_per_block 32..1024, a power of two (default 256; an upper bound
+ *                     for ELL held by diagonals, at most 256, and for CSR with
+ *                     1 or 2 lanes on very uneven rows, at most 128).
  *   threads_per_row   CSR: lanes cooperating on one row, 1/2/4/8/16/32, or
  *                     SPMV_TPR_SPLIT for the nnz-balanced split (default:
  *                     the largest power of two up to 32 that leaves each
@@ -118,13 +123,15 @@ typedef enum {
  *                     1 or 2 lanes on very uneven rows) or items per lane / 4
  *                     (COO, HYB tail, split CSR; at most 16 items).  0 =
  *                     default: ELL and HYB 2 with fp64 values, 4 with
- *                     fp32/bf16; SELL 8 (1 with fp64 values in the
+ *                     fp32/bf16 (held by diagonals: 4, with 16 or more
+ *                     diagonals a slice 8 for fp32 and 1 for bf16); SELL 8 (1 with fp64 values in the
  *                     column-major layout); every other format 2.
  *   regcap            register cap per thread, 32 (the paper's
  *                     maxrregcount knob) or 64 (the ceiling that keeps
  *                     1024-thread blocks launchable); 48 also for ELL, HYB
  *                     and SELL.  0 = default: 32 for ELL and HYB with fp64
- *                     values, 64 otherwise.
+ *                     values, 64 otherwise (held by diagonals: 48 with fp64
+ *                     values, 32 with bf16 and 16 or more a slice).
  *   carveout          preferred shared-memory carveout in percent (0..100),
  *                     or -1 to leave the driver default (Section 4 item 3).
  *                     Zero means 0 % (maximum L1), not "default".

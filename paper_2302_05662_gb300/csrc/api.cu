@@ -248,6 +248,22 @@ int resolve_config(const spmv_matrix *h, const spmv_config *in, spmv_config *out
     return SPMV_OK;
 }
 
+// Unroll and register cap of a handle that keeps diagonals (known once it is
+// packed), where the caller left them at 0.  us at (unroll, cap), 27-point
+// stencil / band of half-width 32 / 5-point: fp64 (2, 32) 112 / 140 / 17.3,
+// (4, 48) 108.5 / 124.8 / 17.3; fp32 (4, 64) 61 / 77 / 13.1, (8, 64) 49 / 50.5 /
+// 15.5; bf16 (4, 64) 37 / 32.7 / 13.3, (1, 32) 32.8 / 32.8 / 18.4.  Slices of
+// few diagonals want them in flight together.
+void dia_defaults(spmv_matrix *h, const spmv_config *in) {
+    if (!h->dia_val || !in) return;
+    const int64_t rows = 32 * dia_rows(h->vt), nslices = (h->m + rows - 1) / rows;
+    const bool few = h->dia_total < 16 * nslices;
+    const int unroll = h->vt == SPMV_F64 || few ? 4 : h->vt == SPMV_F32 ? 8 : 1;
+    const int cap = h->vt == SPMV_F64 ? 48 : h->vt == SPMV_F32 || few ? 64 : 32;
+    if (in->unroll == 0) h->cfg.unroll = unroll;
+    if (in->regcap == 0) h->cfg.regcap = cap;
+}
+
 int runner(const spmv_matrix *h, int kind, double alpha, const void *x, double beta, void *y, cudaStream_t s) {
     switch (h->vt) {
     case SPMV_F64: return run_kernels_f64(kind, h, alpha, x, beta, y, s);
@@ -450,6 +466,7 @@ int spmv_create(spmv_handle *out, int64_t m, int64_t n, int64_t nnz, const int32
     spmv_config rc;
     if (st == SPMV_OK) st = resolve_config(h, cfg, &rc);
     if (st == SPMV_OK) st = pack_format(h, rc, s);
+    if (st == SPMV_OK) dia_defaults(h, cfg);
     if (st != SPMV_OK) {
         destroy_all(h);
         delete h;
@@ -485,6 +502,7 @@ int spmv_set_config(spmv_handle h, const spmv_config *cfg, void *stream) {
         return st;
     }
     int st = pack_format(h, rc, (cudaStream_t)stream);
+    if (st == SPMV_OK) dia_defaults(h, cfg);
     if (st != SPMV_OK) {
         // leave a usable handle: fall back to plain CSR
         spmv_config csr;
@@ -508,6 +526,15 @@ int spmv_get_config(spmv_handle h, spmv_config *out) {
     }
     *out = h->cfg;
     return SPMV_OK;
+}
+
+static int64_t ell_bytes(const spmv_matrix *h) {
+    const int64_t vs = (int64_t)value_size(h->vt), R = dia_rows(h->vt);
+    if (h->dia_val) {
+        const int64_t nslices = (h->m + 32 * R - 1) / (32 * R);
+        return h->dia_total * (32 * R * vs + 4 + 4 * R) + 4 * (nslices + 1);
+    }
+    return h->ell_width * h->ell_pitch * (vs + (h->ell_d16 ? 2 : 4));
 }
 
 int spmv_get_info(spmv_handle h, spmv_info *out) {
@@ -549,7 +576,7 @@ int spmv_get_info(spmv_handle h, spmv_info *out) {
         break;
     case SPMV_FMT_ELL:
         out->ell_width = h->ell_width;
-        out->format_bytes = h->ell_width * h->ell_pitch * (vs + (h->ell_d16 ? 2 : 4));
+        out->format_bytes = ell_bytes(h);
         break;
     case SPMV_FMT_COO:
         out->format_bytes = h->nnz * (vs + 8);
@@ -557,7 +584,7 @@ int spmv_get_info(spmv_handle h, spmv_info *out) {
     case SPMV_FMT_HYB:
         out->ell_width = h->ell_width;
         out->hyb_coo_nnz = h->hyb_nnz;
-        out->format_bytes = h->ell_width * h->ell_pitch * (vs + (h->ell_d16 ? 2 : 4)) + h->hyb_nnz * (vs + 8);
+        out->format_bytes = ell_bytes(h) + h->hyb_nnz * (vs + 8);
         break;
     case SPMV_FMT_BSR:
         out->bsr_blocks = h->bsr_blocks;
@@ -604,10 +631,10 @@ int array_of(spmv_handle h, int32_t id, const void **ptr, int64_t *bytes) {
     case SPMV_ARR_CSR_COLIDX: *ptr = h->colidx; *bytes = 4 * h->nnz; break;
     case SPMV_ARR_CSR_VALS: *ptr = h->vals; *bytes = vs * h->nnz; break;
     case SPMV_ARR_ELL_COLIDX:
-        if (h->ell_col || h->ell_d16) { *ptr = h->ell_col; *bytes = 4 * h->ell_width * h->ell_pitch; }
+        if (h->ell_col || h->ell_d16 || h->dia_val) { *ptr = h->ell_col; *bytes = 4 * h->ell_width * h->ell_pitch; }
         break;
     case SPMV_ARR_ELL_VALS:
-        if (h->ell_val) { *ptr = h->ell_val; *bytes = vs * h->ell_width * h->ell_pitch; }
+        if (h->ell_val || h->dia_val) { *ptr = h->ell_val; *bytes = vs * h->ell_width * h->ell_pitch; }
         break;
     case SPMV_ARR_COO_ROWS:
         if (hyb) { *ptr = h->hyb_rows; *bytes = 4 * h->hyb_nnz; }
@@ -681,6 +708,10 @@ int spmv_export(spmv_handle h, int32_t array_id, void *d_dst, int64_t bytes, voi
         set_error("spmv_export: NULL destination");
         return SPMV_ERR_INVALID;
     }
+    if (array_id == SPMV_ARR_ELL_COLIDX && h->dia_val)  // diagonals: the documented layout, from CSR
+        return export_dia_as_ell(h, static_cast<int32_t *>(d_dst), nullptr, (cudaStream_t)stream);
+    if (array_id == SPMV_ARR_ELL_VALS && h->dia_val)
+        return export_dia_as_ell(h, nullptr, d_dst, (cudaStream_t)stream);
     if (array_id == SPMV_ARR_ELL_COLIDX && h->ell_d16)  // 16-bit row offsets: export int32 columns
         return decode_ell_columns(h, static_cast<int32_t *>(d_dst), (cudaStream_t)stream);
     SPMV_CUDA_TRY(cudaMemcpyAsync(d_dst, p, (size_t)have, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));

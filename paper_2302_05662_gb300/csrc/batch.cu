@@ -67,6 +67,11 @@ struct BatchMat {
     const int16_t *ell_d16;
     const void *ell_val;
     int64_t ell_width, ell_pitch;
+    // ... or the diagonals of slices of 32 dia_r rows
+    const int *dia_ptr, *dia_off;
+    const uint32_t *dia_mask;
+    const void *dia_val;
+    int64_t dia_r;
     // SELL: the handle's work items, arrays and partials; rows from slice
     // s_zero on are empty
     const int *it_slice, *it_base, *it_len, *it_c0, *it_c1;
@@ -88,6 +93,7 @@ constexpr int BATCH_BSR = -SPMV_FMT_BSR;
 // work items of one matrix: CSR split or COO chunks, or 32-row groups, ELL
 // 32-row groups, SELL items plus 32-row groups of its empty rows
 int64_t batch_items(const BatchMat &M, int C) {
+    if (M.fmt == SPMV_FMT_ELL && M.dia_val) return (M.m + 32 * M.dia_r - 1) / (32 * M.dia_r);
     if (M.fmt == SPMV_FMT_ELL) return (M.m + 31) / 32;
     if (M.fmt == SPMV_FMT_SELL) return M.nitems + (std::max<int64_t>(0, M.m - 32 * M.s_zero) + 31) / 32;
     if (M.fmt == SPMV_FMT_BSR) return (M.bsr_mb + 32 / M.bsr_r - 1) / (32 / M.bsr_r);
@@ -122,8 +128,13 @@ void describe_format(const spmv_matrix *h, BatchMat &M) {
         M.bsr_r = h->bsr_r;
     }
     M.n = h->n;
-    if (h->cfg.format == SPMV_FMT_ELL && (h->ell_col || h->ell_d16)) {
+    if (h->cfg.format == SPMV_FMT_ELL && (h->ell_col || h->ell_d16 || h->dia_val)) {
         M.fmt = SPMV_FMT_ELL;
+        M.dia_ptr = h->dia_ptr;
+        M.dia_off = h->dia_off;
+        M.dia_mask = h->dia_mask;
+        M.dia_val = h->dia_val;
+        M.dia_r = dia_rows(h->vt);
         M.ell_col = h->ell_col;
         M.ell_d16 = h->ell_d16;
         M.ell_val = h->ell_val;
@@ -183,7 +194,9 @@ k_batch(const BatchMat *__restrict__ mats, int count, const int64_t *__restrict_
         const T *x = (const T *)M.x;
         T *y = (T *)M.y;
         for (int64_t local = u0; local < u1; ++local) {
-        if (M.fmt == SPMV_FMT_ELL) {  // 32 rows, one per lane
+        if (M.fmt == SPMV_FMT_ELL && M.dia_val) {  // a slice of diagonals
+            dia_slice<V, T, 2>(local, M.m, M.dia_ptr, M.dia_off, M.dia_mask, (const V *)M.dia_val, x, y, ep);
+        } else if (M.fmt == SPMV_FMT_ELL) {  // 32 rows, one per lane
             const int64_t r = local * 32 + lane;
             if (r < M.m) {
                 if (M.ell_d16)
@@ -313,7 +326,7 @@ void free_device(spmv_batch *b) {
 int build(spmv_batch *b, cudaStream_t s) {
     free_device(b);
     const int C = 32 * b->items;
-    std::vector<BatchMat> mats(b->count);
+    std::vector<BatchMat> mats(b->count, BatchMat{});
     std::vector<int64_t> off(b->count + 1, 0);
     b->metas.assign(b->count, nullptr);
     int64_t chunks_total = 0;

@@ -41,6 +41,23 @@ __global__ void k_check_d16(const int16_t *a, int64_t width, int64_t pitch, int6
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, STATUS_BOUNDS);
 }
 
+// ELL by diagonals: every row with a bit on a diagonal has its column in [0, n)
+__global__ void k_check_dia(const int *ptr, const int *off, const uint32_t *mask, int R, int64_t nslices, int64_t m,
+                            int64_t n, unsigned *status) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    bool bad = false;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nslices * 32 * R; t += stride) {
+        const int64_t sl = t / (32 * R), row = t;
+        const int i = (int)(t % (32 * R)) / 32, l = (int)(t % 32);
+        for (int d = ptr[sl]; d < ptr[sl + 1]; ++d)
+            if ((mask[(int64_t)d * R + i] >> l) & 1u) {
+                const int64_t c = row + off[d];
+                if (row >= m || c < 0 || c >= n) bad = true;
+            }
+    }
+    if (bad) atomicOr(status, STATUS_BOUNDS);
+}
+
 // row pointers: p[0] == 0, nondecreasing, p[rows] == total
 __global__ void k_check_ptr(const int *p, int64_t rows, int64_t total, unsigned *status) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -76,7 +93,12 @@ int check_indices(const spmv_matrix *h, cudaStream_t s) {
     switch (h->cfg.format) {
     case SPMV_FMT_ELL:
     case SPMV_FMT_HYB:
-        if (h->ell_d16)
+        if (h->dia_val) {
+            const int R = dia_rows(h->vt);
+            const int64_t nslices = (m + 32 * R - 1) / (32 * R);
+            k_check_ptr<<<grid_for(nslices + 1), 256, 0, s>>>(h->dia_ptr, nslices, h->dia_total, st);
+            k_check_dia<<<grid_for(m), 256, 0, s>>>(h->dia_ptr, h->dia_off, h->dia_mask, R, nslices, m, n, st);
+        } else if (h->ell_d16)
             k_check_d16<<<grid_for(h->ell_width * h->ell_pitch), 256, 0, s>>>(h->ell_d16, h->ell_width, h->ell_pitch,
                                                                              m, n, st);
         else if (h->ell_col)

@@ -6,6 +6,7 @@
 // merging of duplicate pairs, the row-pointer array, and the packs of the
 // other formats from CSR (Section 2.3 layouts).
 #include <algorithm>
+#include <climits>
 #include <vector>
 
 #include "combine.cuh"
@@ -746,6 +747,113 @@ __global__ void __launch_bounds__(128) k_ell_pack(const int *__restrict__ rowptr
     }
 }
 
+// Diagonals of a slice (32 R rows, of each row its first `width` entries): a
+// merge of the rows' ascending offsets, one step per distinct offset.  Without
+// FILL the steps are counted (given up past `most`), with FILL each step
+// writes its offset, row masks and values.  One warp per slice, every
+// step_s-th slice; the slice's columns and values are staged as in k_ell_pack.
+template <typename V, int R, bool FILL>
+__global__ void __launch_bounds__(128)
+k_dia_slices(const int *__restrict__ rowptr, const int *__restrict__ colidx, const V *__restrict__ vals, int64_t m,
+             int64_t width, int64_t nslices, int64_t step_s, int most, int cap, const int *__restrict__ ptr, int *count,
+             unsigned long long *sums, int *off, uint32_t *mask, V *val) {
+    extern __shared__ __align__(16) unsigned char pack_smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const size_t words = ell_pack_words(cap);
+    V *sv = reinterpret_cast<V *>(pack_smem) + warp * words;
+    int *sc = FILL ? reinterpret_cast<int *>(pack_smem + (sizeof(V) * words * nw + 15) / 16 * 16) + warp * words
+                   : reinterpret_cast<int *>(pack_smem) + warp * words;
+    unsigned diags = 0, entries = 0;
+    for (int64_t sl = ((int64_t)blockIdx.x * nw + warp) * step_s; sl < nslices; sl += (int64_t)gridDim.x * nw * step_s) {
+        int p[R], e[R], d[R];
+        int64_t row[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            row[i] = sl * (32 * R) + 32 * i + lane;
+            p[i] = __ldg(rowptr + (row[i] < m ? row[i] : m));
+            e[i] = __ldg(rowptr + (row[i] + 1 < m ? row[i] + 1 : m));
+        }
+        const int w0 = __shfl_sync(FULL, p[0], 0), w1 = __shfl_sync(FULL, e[R - 1], 31);
+        const bool staged = w1 - w0 <= cap;
+        __syncwarp();
+        if (staged) {
+#pragma unroll 8
+            for (int o = lane; o < w1 - w0; o += 32) {
+                sc[o + (o >> 5)] = __ldg(colidx + w0 + o);
+                if (FILL) sv[o + (o >> 5)] = vals[w0 + o];
+            }
+        }
+        __syncwarp();
+        auto col = [&](int k) -> int { return staged ? sc[(k - w0) + ((k - w0) >> 5)] : __ldg(colidx + k); };
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            if (e[i] - p[i] > width) e[i] = p[i] + (int)width;
+            entries += e[i] - p[i];
+            d[i] = p[i] < e[i] ? (int)(col(p[i]) - row[i]) : INT_MAX;
+        }
+        int64_t at = FILL ? __ldg(ptr + sl) : 0;
+        int n = 0;
+        for (;;) {
+            int lo = d[0];
+#pragma unroll
+            for (int i = 1; i < R; ++i) lo = min(lo, d[i]);
+            lo = __reduce_min_sync(FULL, lo);
+            if (lo == INT_MAX || (!FILL && n == most)) break;
+            V v[R];
+            uint32_t w[R];
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const bool hit = d[i] == lo;
+                if (FILL) {
+                    w[i] = __ballot_sync(FULL, hit);
+                    v[i] = V(0.0f);
+                    if (hit) v[i] = staged ? sv[(p[i] - w0) + ((p[i] - w0) >> 5)] : vals[p[i]];
+                }
+                if (hit) {
+                    ++p[i];
+                    d[i] = p[i] < e[i] ? (int)(col(p[i]) - row[i]) : INT_MAX;
+                }
+            }
+            if (FILL) {
+                if (lane == 0) {
+                    off[at] = lo;
+#pragma unroll
+                    for (int i = 0; i < R; ++i) mask[at * R + i] = w[i];
+                }
+#pragma unroll
+                for (int i = 0; i < R; ++i) val[(at * 32 + lane) * R + i] = v[i];
+                ++at;
+            }
+            ++n;
+        }
+        if (!FILL) {
+            if (lane == 0 && count) count[sl] = n;
+            diags += n;
+        }
+    }
+    if (!FILL) {
+        entries = __reduce_add_sync(FULL, entries);
+        if (lane == 0) {
+            atomicAdd(sums, (unsigned long long)diags);
+            atomicAdd(sums + 1, (unsigned long long)entries);
+        }
+    }
+}
+
+// rows of the diagonal layout as ELL columns and values (either may be null)
+template <typename V>
+__global__ void k_ell_from_csr(const int *rowptr, const int *colidx, const V *vals, int64_t m, int64_t width,
+                               int64_t pitch, int *cols, V *out) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < pitch; r += stride) {
+        const int s = r < m ? rowptr[r] : 0, len = r < m ? rowptr[r + 1] - s : 0;
+        for (int64_t k = 0; k < width; ++k) {
+            if (cols) cols[k * pitch + r] = k < len ? colidx[s + k] : -1;
+            if (out) out[k * pitch + r] = k < len ? vals[s + k] : V(0.0f);
+        }
+    }
+}
+
 // largest |column - row| of the matrix (columns ascend within a row, so a
 // row's first and last entries bound it)
 __global__ void k_max_offset(const int *rowptr, const int *colidx, int64_t m, int *out) {
@@ -1116,6 +1224,21 @@ int decode_ell_columns(const spmv_matrix *h, int32_t *d_out, cudaStream_t s) {
     return SPMV_OK;
 }
 
+// the ELL arrays of a handle that keeps diagonals, in the documented layout
+int export_dia_as_ell(spmv_matrix *h, int32_t *cols, void *vals, cudaStream_t s) {
+    const unsigned g = grid1d(h->ell_pitch, 256);
+    auto go = [&](auto *v) {
+        using V = std::remove_pointer_t<decltype(v)>;
+        k_ell_from_csr<V><<<g, 256, 0, s>>>(h->rowptr, h->colidx, (const V *)h->vals, h->m, h->ell_width, h->ell_pitch,
+                                            cols, (V *)vals);
+    };
+    if (h->vt == SPMV_F64) go((double *)nullptr);
+    else if (h->vt == SPMV_F32) go((float *)nullptr);
+    else go((__nv_bfloat16 *)nullptr);
+    SPMV_CUDA_TRY(cudaGetLastError());
+    return SPMV_OK;
+}
+
 int expand_rows(const int32_t *rowptr, int64_t m, int64_t nnz, int32_t *rows_out, cudaStream_t s) {
     if (nnz == 0) return SPMV_OK;
     k_expand_rows<<<grid1d(nnz, 256), 256, 0, s>>>(rowptr, m, nnz, rows_out);
@@ -1360,6 +1483,11 @@ void free_packed(spmv_matrix *h) {
     f(h->ell_col); h->ell_col = nullptr;
     f(h->ell_d16); h->ell_d16 = nullptr;
     f(h->ell_val); h->ell_val = nullptr;
+    f(h->dia_ptr); h->dia_ptr = nullptr;
+    f(h->dia_off); h->dia_off = nullptr;
+    f(h->dia_mask); h->dia_mask = nullptr;
+    f(h->dia_val); h->dia_val = nullptr;
+    h->dia_total = 0;
     h->ell_width = h->ell_pitch = 0;
     f(h->hyb_rows); h->hyb_rows = nullptr;
     f(h->hyb_cols); h->hyb_cols = nullptr;
@@ -1405,6 +1533,76 @@ int launch_ell_pack(spmv_matrix *h, int64_t width, int64_t pitch, CI *cols, cuda
     return launch_ell_pack_t<__nv_bfloat16, CI>(h, width, pitch, cols, s);
 }
 
+// Diagonals instead of columns, where that makes the product read clearly
+// fewer bytes: at most 0.8 of the column-major layout's, and with fp64 values
+// (one multiply-add per slot of a diagonal, entry or not, on the pipe that
+// bounds them) at most 1.06 slots per entry; and from 2^20 entries on: smaller
+// matrices stay in L2, where a product lasts as long as its launch either way.
+// A sample of 256 slices says whether it is worth counting them all.  *done:
+// the handle keeps diagonals.
+template <typename V>
+int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, bool *done) {
+    constexpr int R = DIA_ROWS<V>;
+    *done = false;
+    const int64_t m = h->m, nslices = (m + 32 * R - 1) / (32 * R);
+    if (width == 0 || h->nnz < (1 << 20)) return SPMV_OK;
+    const int cap = (int)std::min<int64_t>(ELL_PACK_CAP, 32 * R * width);
+    auto shape = [&](size_t entry_bytes, int *nw, size_t *smem) {
+        const size_t per_warp = ell_pack_words(cap) * entry_bytes;
+        *nw = (int)std::max<size_t>(1, std::min<size_t>(4, ELL_PACK_SMEM / per_warp));
+        *smem = per_warp * *nw + 16;
+    };
+    int nw;
+    size_t smem;
+    Tmp<unsigned long long> sums;
+    Tmp<int> count;
+    SPMV_TRY(sums.alloc(2, s));
+    auto count_kernel = k_dia_slices<V, R, false>;
+    shape(4, &nw, &smem);
+    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the diagonals of `slices` slices (one in step_s) and the entries on them
+    auto counted = [&](int64_t step_s, int *out, bool *worth) -> int {
+        const int64_t slices = (nslices + step_s - 1) / step_s;
+        unsigned long long hs[2];
+        SPMV_CUDA_TRY(cudaMemsetAsync(sums.p, 0, sizeof(hs), s));
+        count_kernel<<<grid1d(slices, nw, 1 << 20), 32 * nw, smem, s>>>(
+            h->rowptr, h->colidx, (const V *)h->vals, m, width, nslices, step_s, (int)std::min<int64_t>(4 * width + 16, 1 << 20),
+            cap, nullptr, out, sums.p, nullptr, nullptr, nullptr);
+        SPMV_CUDA_TRY(cudaGetLastError());
+        SPMV_CUDA_TRY(cudaMemcpyAsync(hs, sums.p, sizeof(hs), cudaMemcpyDeviceToHost, s));
+        SPMV_CUDA_TRY(cudaStreamSynchronize(s));
+        const double slots = 32.0 * R * (double)hs[0], entries = (double)hs[1];
+        const double dia = slots * sizeof(V) + (double)hs[0] * (4 + 4 * R), ell = entries * (double)(sizeof(V) + index_bytes);
+        *worth = entries > 0 && dia <= 0.8 * ell && (sizeof(V) < 8 || slots <= 1.06 * entries);
+        return SPMV_OK;
+    };
+    bool worth = false;
+    if (nslices > 512) {
+        SPMV_TRY(counted(nslices / 256, nullptr, &worth));
+        if (!worth) return SPMV_OK;
+    }
+    SPMV_TRY(count.alloc(nslices + 1, s));
+    SPMV_CUDA_TRY(cudaMemsetAsync(count.p + nslices, 0, sizeof(int), s));
+    SPMV_TRY(counted(1, count.p, &worth));
+    if (!worth) return SPMV_OK;
+    int64_t total = 0;
+    SPMV_TRY(dalloc(&h->dia_ptr, (size_t)nslices + 1));
+    SPMV_TRY(exclusive_scan(count.p, h->dia_ptr, nslices + 1, s, &total));
+    h->dia_total = total;
+    SPMV_TRY(dalloc(&h->dia_off, (size_t)total));
+    SPMV_TRY(dalloc(&h->dia_mask, (size_t)total * R));
+    SPMV_TRY(dalloc_bytes(&h->dia_val, sizeof(V) * (size_t)total * 32 * R));
+    auto fill = k_dia_slices<V, R, true>;
+    shape(4 + sizeof(V), &nw, &smem);
+    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    fill<<<grid1d(nslices, nw, 1 << 20), 32 * nw, smem, s>>>(h->rowptr, h->colidx, (const V *)h->vals, m, width, nslices, 1,
+                                                             INT_MAX, cap, h->dia_ptr, nullptr, nullptr, h->dia_off,
+                                                             h->dia_mask, (V *)h->dia_val);
+    SPMV_CUDA_TRY(cudaGetLastError());
+    *done = true;
+    return SPMV_OK;
+}
+
 // bf16 values: columns are stored as 16-bit offsets from the row when
 // every |column - row| of the matrix is at most 32767 (stencils, banded and
 // block-diagonal matrices), 2 index bytes per slot instead of 4.  Measured
@@ -1413,7 +1611,7 @@ int launch_ell_pack(spmv_matrix *h, int64_t width, int64_t pitch, CI *cols, cuda
 // default 4; fp64 loses 8-10% (its ELL kernel is held by the fp64 pipe and
 // the decode sits between the column load and the x gather).  fp32 and
 // fp64 keep int32 columns.
-int pack_ell(spmv_matrix *h, int64_t width, bool hyb, cudaStream_t s) {
+int pack_ell(spmv_matrix *h, int64_t width, cudaStream_t s) {
     const int64_t m = h->m;
     const int64_t pitch = (m + 31) / 32 * 32;
     const size_t vs = value_size(h->vt);
@@ -1429,6 +1627,12 @@ int pack_ell(spmv_matrix *h, int64_t width, bool hyb, cudaStream_t s) {
         SPMV_CUDA_TRY(cudaMemcpyAsync(&maxoff, mo.p, sizeof(int), cudaMemcpyDeviceToHost, s));
         SPMV_CUDA_TRY(cudaStreamSynchronize(s));
     }
+    bool dia = false;
+    const int index_bytes = maxoff <= 32767 ? 2 : 4;
+    if (h->vt == SPMV_F64) SPMV_TRY(pack_dia<double>(h, width, index_bytes, s, &dia));
+    else if (h->vt == SPMV_F32) SPMV_TRY(pack_dia<float>(h, width, index_bytes, s, &dia));
+    else SPMV_TRY(pack_dia<__nv_bfloat16>(h, width, index_bytes, s, &dia));
+    if (dia) return SPMV_OK;
     SPMV_TRY(dalloc_bytes(&h->ell_val, vs * width * pitch));
     if (maxoff <= 32767) {
         SPMV_TRY(dalloc(&h->ell_d16, (size_t)(width * pitch)));
@@ -1437,7 +1641,6 @@ int pack_ell(spmv_matrix *h, int64_t width, bool hyb, cudaStream_t s) {
         SPMV_TRY(dalloc(&h->ell_col, (size_t)(width * pitch)));
         if (width > 0 && pitch > 0) SPMV_TRY(launch_ell_pack<int>(h, width, pitch, h->ell_col, s));
     }
-    (void)hyb;
     return SPMV_OK;
 }
 
@@ -1467,7 +1670,7 @@ int hyb_width_rule(spmv_matrix *h, cudaStream_t s, int64_t *width) {
 
 int pack_hyb(spmv_matrix *h, int64_t width, cudaStream_t s) {
     const int64_t m = h->m;
-    SPMV_TRY(pack_ell(h, width, true, s));
+    SPMV_TRY(pack_ell(h, width, s));
     SPMV_TRY(dalloc(&h->hyb_ptr, (size_t)m + 1));
     Tmp<int> cnt;
     SPMV_TRY(cnt.alloc(m + 1, s));
@@ -1735,7 +1938,7 @@ int pack_format(spmv_matrix *h, const spmv_config &cfg, cudaStream_t s) {
                       (long long)pitch);
             return SPMV_ERR_UNSUPPORTED;
         }
-        SPMV_TRY(pack_ell(h, width, false, s));
+        SPMV_TRY(pack_ell(h, width, s));
         break;
     }
     case SPMV_FMT_COO:

@@ -62,6 +62,10 @@ template <> struct VT_<SPMV_BF16> { using V = __nv_bfloat16; using T = float; };
 inline size_t value_size(int vt) { return vt == SPMV_F64 ? 8 : vt == SPMV_F32 ? 4 : 2; }
 inline size_t vec_size(int vt) { return vt == SPMV_F64 ? 8 : 4; }
 
+// rows per lane of a slice of diagonals: 8 bytes of values per lane and load
+template <typename V> constexpr int DIA_ROWS = 8 / sizeof(V);
+inline int dia_rows(int vt) { return (int)(8 / value_size(vt)); }
+
 // ---------------------------------------------------------------------------
 // device load helpers.  Matrix arrays are streamed once per product: they
 // are read through the non-coherent path without L1 allocation so that L1
@@ -324,6 +328,16 @@ struct spmv_matrix {
     int32_t *ell_col = nullptr;   // int32 columns, padding -1 ...
     int16_t *ell_d16 = nullptr;   // ... or 16-bit column - row, padding INT16_MIN
     void *ell_val = nullptr;
+    // ... or, where the rows of a slice (32 dia_rows(vt) rows) share their
+    // column - row offsets, diagonals of each slice instead of the three
+    // arrays above: slice s holds diagonals [dia_ptr[s], dia_ptr[s+1]),
+    // ascending; diagonal d has one offset, a bit per row that holds an entry
+    // there (dia_rows words, word i bit l: row 32 i + l), and a value per row
+    // (0 without an entry) at (32 d + l) dia_rows + i
+    int64_t dia_total = 0;
+    int32_t *dia_ptr = nullptr, *dia_off = nullptr;
+    uint32_t *dia_mask = nullptr;
+    void *dia_val = nullptr;
     // HYB COO part
     int64_t hyb_nnz = 0;
     int32_t *hyb_rows = nullptr, *hyb_cols = nullptr, *hyb_ptr = nullptr;
@@ -366,6 +380,7 @@ void free_packed(spmv_matrix *h);
 int expand_rows(const int32_t *rowptr, int64_t m, int64_t nnz, int32_t *rows_out,
                 cudaStream_t s);
 int decode_ell_columns(const spmv_matrix *h, int32_t *d_out, cudaStream_t s);
+int export_dia_as_ell(spmv_matrix *h, int32_t *cols, void *vals, cudaStream_t s);
 // chunk metadata kinds: COO / HYB tail, staged CSR tiles, CSR warp chunks
 enum { SEG_COO = 0, SEG_TILES = 1, SEG_MERGE = 2 };
 int ensure_seg_scratch(spmv_matrix *h, int items, int kind, cudaStream_t s);

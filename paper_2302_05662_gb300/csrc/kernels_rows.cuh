@@ -461,6 +461,131 @@ k_ell2(int64_t m, int64_t width, int64_t pitch, const CI *__restrict__ col, cons
 }
 
 // ---------------------------------------------------------------------------
+// ELL by diagonals (stencils, bands): where the rows of a slice share their
+// column - row offsets, a diagonal of the slice stores one offset and a row
+// mask instead of a column per slot, so a slot is its value alone (bf16 band
+// of half-width 32: 4 bytes a slot with 16-bit offsets, 2.1 here), the gathers
+// of x are contiguous, and their addresses do not wait for a column load.  A
+// warp takes a slice, lane l the rows l, l + 32, ...; a row's entries come in
+// ascending column order, as in the column-major layout.  The offsets and
+// masks of 32 diagonals are held by the lanes and handed round by shuffles.
+// Measured, column-major / diagonals, us: 27-point stencil 128^3 fp64 113.5 /
+// 108.5, fp32 79.6 / 49.0, bf16 57.6 / 32.9; band of half-width 32, 2^20 rows,
+// fp64 133.8 / 124.8, fp32 95.1 / 50.5, bf16 64.6 / 32.8.  The fp64 forms are
+// bound by the fp64 pipe (105 and 129 by the FMA rate of the probe), the
+// others by load latency at 70 to 85% of their bytes at the HBM rate.
+// ---------------------------------------------------------------------------
+template <int R> struct MaskWords;
+template <> struct MaskWords<1> {
+    static __device__ __forceinline__ void load(const uint32_t *p, uint32_t (&o)[1]) { o[0] = __ldg(p); }
+};
+template <> struct MaskWords<2> {
+    static __device__ __forceinline__ void load(const uint32_t *p, uint32_t (&o)[2]) {
+        const uint2 w = __ldg(reinterpret_cast<const uint2 *>(p));
+        o[0] = w.x; o[1] = w.y;
+    }
+};
+template <> struct MaskWords<4> {
+    static __device__ __forceinline__ void load(const uint32_t *p, uint32_t (&o)[4]) {
+        const uint4 w = __ldg(reinterpret_cast<const uint4 *>(p));
+        o[0] = w.x; o[1] = w.y; o[2] = w.z; o[3] = w.w;
+    }
+};
+// a lane's values of one diagonal (8 bytes)
+__device__ __forceinline__ void ld_dia(const double *p, double (&o)[1]) { o[0] = ld_s(p); }
+__device__ __forceinline__ void ld_dia(const float *p, float (&o)[2]) {
+    const float2 w = ld_s(reinterpret_cast<const float2 *>(p));
+    o[0] = w.x; o[1] = w.y;
+}
+__device__ __forceinline__ void ld_dia(const __nv_bfloat16 *p, float (&o)[4]) {
+    const uint2 w = ld_s(reinterpret_cast<const uint2 *>(p));
+    o[0] = bf16lo(w.x); o[1] = bf16hi(w.x); o[2] = bf16lo(w.y); o[3] = bf16hi(w.y);
+}
+
+// U diagonals from the warp's k-th on, in flight together.  A row without an
+// entry on a diagonal loads no x: its slot's value is 0 and its x is taken as 0.
+template <int U, typename V, typename T, int R>
+__device__ __forceinline__ void dia_step(int k, const V *__restrict__ vp, int o, const uint32_t (&w)[R], uint32_t full,
+                                         const T *__restrict__ xr, T (&acc)[R]) {
+    const int lane = threadIdx.x & 31;
+    T v[U][R], xv[U][R];
+#pragma unroll
+    for (int u = 0; u < U; ++u) ld_dia(vp + (int64_t)(k + u) * (32 * R), v[u]);
+    constexpr uint32_t SOME = (1u << U) - 1u;
+    if (((full >> k) & SOME) == SOME) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const T *xd = xr + __shfl_sync(FULLMASK, o, k + u);
+#pragma unroll
+            for (int i = 0; i < R; ++i) xv[u][i] = __ldg(xd + 32 * i);
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const T *xd = xr + __shfl_sync(FULLMASK, o, k + u);
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const uint32_t bits = __shfl_sync(FULLMASK, w[i], k + u);
+                xv[u][i] = T(0);
+                if ((bits >> lane) & 1u) xv[u][i] = __ldg(xd + 32 * i);
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int i = 0; i < R; ++i) acc[i] = fma(v[u][i], xv[u][i], acc[i]);
+}
+
+// one slice; the whole warp calls it, U diagonals in flight
+template <typename V, typename T, int U>
+__device__ __forceinline__ void dia_slice(int64_t sl, int64_t m, const int *__restrict__ ptr, const int *__restrict__ off,
+                                          const uint32_t *__restrict__ mask, const V *__restrict__ val,
+                                          const T *__restrict__ x, T *__restrict__ y, const Epi<T> &ep) {
+    constexpr int R = DIA_ROWS<V>;
+    const int lane = threadIdx.x & 31;
+    const int p0 = __ldg(ptr + sl), p1 = __ldg(ptr + sl + 1);
+    const int64_t r0 = sl * (32 * R) + lane;
+    const T *xr = x + r0;  // entry of row r0 + 32 i on a diagonal of offset o: xr[o + 32 i]
+    T acc[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) acc[i] = T(0);
+    for (int p = p0; p < p1; p += 32) {
+        const int cnt = p1 - p < 32 ? p1 - p : 32;
+        int o = 0;
+        uint32_t w[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) w[i] = 0u;
+        if (lane < cnt) {
+            o = __ldg(off + p + lane);
+            MaskWords<R>::load(mask + (int64_t)(p + lane) * R, w);
+        }
+        bool all = true;
+#pragma unroll
+        for (int i = 0; i < R; ++i) all = all && w[i] == FULLMASK;
+        const uint32_t full = __ballot_sync(FULLMASK, all);  // diagonals every row of the slice is on
+        const V *vp = val + ((int64_t)p * 32 + lane) * R;
+        int k = 0;
+        for (; k + U <= cnt; k += U) dia_step<U>(k, vp, o, w, full, xr, acc);
+        for (; k < cnt; ++k) dia_step<1>(k, vp, o, w, full, xr, acc);
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+        if (r0 + 32 * i < m) ep.store(y, r0 + 32 * i, acc[i]);
+}
+
+template <typename V, typename T, int U, int REGCAP>
+__global__ void __launch_bounds__(1024) __maxnreg__(REGCAP)
+k_ell_dia(int64_t m, int64_t nslices, const int *__restrict__ ptr, const int *__restrict__ off,
+          const uint32_t *__restrict__ mask, const V *__restrict__ val, const T *__restrict__ x, T *__restrict__ y,
+          T alpha, T beta) {
+    const Epi<T> ep(alpha, beta);
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t sl = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; sl < nslices; sl += nwarps)
+        dia_slice<V, T, U>(sl, m, ptr, off, mask, val, x, y, ep);
+}
+
+// ---------------------------------------------------------------------------
 // BSR with R x R row-major blocks (the blocked ELL of Section 2.3 stored by
 // block rows).  A group of R*S lanes owns a block row: lane (s, i) takes
 // row i of every S-th block, so a warp reads whole blocks contiguously.

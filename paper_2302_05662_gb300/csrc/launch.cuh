@@ -147,7 +147,24 @@ int launch_ell_ci(const spmv_matrix *h, const CI *cols, int64_t width, T alpha, 
 }
 
 template <typename V, typename T, int U, int RC>
+int launch_ell_dia(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, cudaStream_t s) {
+    auto kern = k_ell_dia<V, T, U, RC>;
+    // slices are independent warps: larger blocks only leave registers unused
+    // (27-point stencil, fp64, 48 registers: 108.5 us with 256 threads, 122.6 with 1024)
+    const int tpb = std::min(256, h->cfg.threads_per_block);
+    SPMV_TRY(apply_carveout((const void *)kern, h->cfg.carveout));
+    constexpr int rows = 32 * DIA_ROWS<V>;
+    const int64_t nslices = (h->m + rows - 1) / rows, wpb = tpb / 32;
+    const int grid = wave_grid((const void *)kern, tpb, (nslices + wpb - 1) / wpb, h->sm_count);
+    kern<<<grid, tpb, 0, s>>>(h->m, nslices, h->dia_ptr, h->dia_off, h->dia_mask, (const V *)h->dia_val, x, y, alpha,
+                              beta);
+    SPMV_LAUNCH_CHECK();
+    return SPMV_OK;
+}
+
+template <typename V, typename T, int U, int RC>
 int launch_ell_rc(const spmv_matrix *h, int64_t width, T alpha, const T *x, T beta, T *y, cudaStream_t s) {
+    if (h->dia_val) return launch_ell_dia<V, T, U, RC>(h, alpha, x, beta, y, s);
     if (h->ell_d16) return launch_ell_ci<V, T, U, RC, int16_t>(h, h->ell_d16, width, alpha, x, beta, y, s);
     return launch_ell_ci<V, T, U, RC, int>(h, h->ell_col, width, alpha, x, beta, y, s);
 }
