@@ -311,12 +311,12 @@ void free_device(spmv_batch *b) {
     if (b->graph) cudaGraphDestroy(b->graph);
     b->exec = nullptr;
     b->graph = nullptr;
-    if (b->d_mats) cudaFree(b->d_mats);
-    if (b->d_item_off) cudaFree(b->d_item_off);
+    dev_free(b->d_mats);
+    dev_free(b->d_item_off);
     b->d_mats = nullptr;
     b->d_item_off = nullptr;
     for (int32_t *p : b->metas)
-        if (p) cudaFree(p);
+        dev_free(p);
     b->metas.clear();
     free_partials(&b->part);
 }
@@ -477,7 +477,7 @@ int spmv_batch_create(spmv_batch_handle *out, const spmv_handle *hs, int32_t cou
     if (st == SPMV_OK) st = build(b, (cudaStream_t)stream);
     if (st != SPMV_OK) {
         free_device(b);
-        if (b->d_counter) cudaFree(b->d_counter);
+        dev_free(b->d_counter);
         if (b->cs) cudaStreamDestroy(b->cs);
         delete b;
         return st;
@@ -594,9 +594,9 @@ int spmv_batch_tune(spmv_batch_handle b, void *stream) {
                 }
             }
             free_partials(&one.part);
-            if (meta) cudaFree(meta);
-            if (d_m) cudaFree(d_m);
-            if (d_off) cudaFree(d_off);
+            dev_free(meta);
+            dev_free(d_m);
+            dev_free(d_off);
             one.d_counter = nullptr;
             one.cs = nullptr;
             if (st != SPMV_OK) return st;
@@ -648,7 +648,7 @@ int spmv_batch_destroy(spmv_batch_handle b) {
     if (!b) return SPMV_OK;
     if (b->cs) cudaStreamSynchronize(b->cs);
     free_device(b);
-    if (b->d_counter) cudaFree(b->d_counter);
+    dev_free(b->d_counter);
     if (b->cs) cudaStreamDestroy(b->cs);
     delete b;
     return SPMV_OK;

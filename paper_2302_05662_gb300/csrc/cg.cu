@@ -555,12 +555,12 @@ void free_cg(spmv_matrix *h) {
     if (c->exec) cudaGraphExecDestroy(c->exec);
     if (c->graph) cudaGraphDestroy(c->graph);
     if (c->cs) cudaStreamDestroy(c->cs);
-    cudaFree(c->r);
-    cudaFree(c->p);
-    cudaFree(c->q);
-    cudaFree(c->part);
-    cudaFree(c->hist);
-    cudaFree(c->st);
+    dev_free(c->r);
+    dev_free(c->p);
+    dev_free(c->q);
+    dev_free(c->part);
+    dev_free(c->hist);
+    dev_free(c->st);
     delete c;
     h->cg = nullptr;
 }

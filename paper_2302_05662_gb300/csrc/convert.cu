@@ -7,6 +7,7 @@
 // other formats from CSR (Section 2.3 layouts).
 #include <algorithm>
 #include <climits>
+#include <initializer_list>
 #include <vector>
 
 #include "combine.cuh"
@@ -60,6 +61,30 @@ inline int bits_for(int64_t count) {  // bits to hold 0 .. count-1
     while ((int64_t(1) << b) < count) ++b;
     return b;
 }
+// One block of several arrays, each on a 256-byte boundary; the first is the
+// owner, the one to free.  (Mapping and unmapping cost by the block as well as
+// by the byte.)
+struct Slab {
+    void **p;
+    size_t bytes;
+};
+int dalloc_slab(std::initializer_list<Slab> parts) {
+    size_t total = 0;
+    for (const Slab &q : parts) total += (std::max<size_t>(q.bytes, 1) + 255) / 256 * 256;
+    char *base = nullptr;
+    for (const Slab &q : parts) *q.p = nullptr;
+    cudaError_t e = dev_malloc(reinterpret_cast<void **>(&base), total);
+    if (e != cudaSuccess) return cuda_status(e, "cudaMalloc");
+    for (const Slab &q : parts) {
+        *q.p = base;
+        base += (std::max<size_t>(q.bytes, 1) + 255) / 256 * 256;
+    }
+    return SPMV_OK;
+}
+template <typename T>
+Slab slab(T **p, size_t count) { return Slab{reinterpret_cast<void **>(p), sizeof(T) * count}; }
+inline Slab slab_bytes(void **p, size_t bytes) { return Slab{p, bytes}; }
+
 inline unsigned grid1d(int64_t work, int threads, int cap = 152 * 32) {
     int64_t g = (work + threads - 1) / threads;
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(g, cap));
@@ -679,8 +704,7 @@ int sort_and_merge(spmv_matrix *h, const int32_t *d_rows, const int32_t *d_cols,
     SPMV_CUDA_TRY(cudaStreamSynchronize(s));
     h->nnz = nu;
     SPMV_TRY(urows->alloc(nu, s));
-    SPMV_TRY(dalloc(&h->colidx, (size_t)nu + CSR_PAD));
-    SPMV_TRY(dalloc_bytes(&h->vals, sizeof(V) * (nu + CSR_PAD)));
+    SPMV_TRY(dalloc_slab({slab_bytes(&h->vals, sizeof(V) * (nu + CSR_PAD)), slab(&h->colidx, (size_t)nu + CSR_PAD)}));
     k_merge_runs<V, T><<<(unsigned)nb, SC_THREADS, 0, s>>>(ks, reinterpret_cast<const V *>(vsorted), sums.p, nnz, colbits,
                                                            urows->p, h->colidx, (V *)h->vals);
     SPMV_CUDA_TRY(cudaGetLastError());
@@ -1356,8 +1380,7 @@ int build_csr(spmv_matrix *h, const int32_t *d_rows, const int32_t *d_cols, cons
     SPMV_TRY(dalloc(&h->rowptr, (size_t)m + 1 + CSR_PAD));  // staged windows may read 3 past m
     if (nnz_in == 0) {
         SPMV_CUDA_TRY(cudaMemsetAsync(h->rowptr, 0, sizeof(int) * (m + 1), s));
-        SPMV_TRY(dalloc(&h->colidx, 1));
-        SPMV_TRY(dalloc_bytes(&h->vals, vs));
+        SPMV_TRY(dalloc_slab({slab_bytes(&h->vals, vs), slab(&h->colidx, 1)}));
         h->max_row = 0;
         SPMV_CUDA_TRY(cudaStreamSynchronize(s));
         return SPMV_OK;
@@ -1390,8 +1413,7 @@ int build_csr(spmv_matrix *h, const int32_t *d_rows, const int32_t *d_cols, cons
     if (!(hflags & 6u)) {
         // already sorted by (row, col) with no repeated pair: copy and index
         h->nnz = nnz_in;
-        SPMV_TRY(dalloc(&h->colidx, (size_t)nnz_in + CSR_PAD));
-        SPMV_TRY(dalloc_bytes(&h->vals, vs * (nnz_in + CSR_PAD)));
+        SPMV_TRY(dalloc_slab({slab_bytes(&h->vals, vs * (nnz_in + CSR_PAD)), slab(&h->colidx, (size_t)nnz_in + CSR_PAD)}));
         SPMV_CUDA_TRY(cudaMemcpyAsync(h->colidx, d_cols, sizeof(int) * nnz_in, cudaMemcpyDeviceToDevice, s));
         SPMV_CUDA_TRY(cudaMemcpyAsync(h->vals, d_vals, vs * nnz_in, cudaMemcpyDeviceToDevice, s));
         if (hflags & 8u) {  // long runs of empty rows: every row pointer by a search
@@ -1437,14 +1459,14 @@ int alloc_partials(Partials *p, int64_t units, int stride, int vt, cudaStream_t 
 }
 
 void free_partials(Partials *p) {
-    auto f = [](void *q) { if (q) cudaFree(q); };
+    auto f = [](void *q) { dev_free(q); };
     f(p->head); f(p->tail); f(p->count); f(p->xslot);
     *p = Partials{};
 }
 
 static void free_long_rows(spmv_matrix *h) {
     LongRows &L = h->lng;
-    auto f = [](void *q) { if (q) cudaFree(q); };
+    auto f = [](void *q) { dev_free(q); };
     f(L.seg_row); f(L.seg_begin); f(L.seg_end); f(L.seg_c0); f(L.seg_c1);
     free_partials(&L.part);
     L = LongRows{};
@@ -1478,15 +1500,15 @@ int build_long_rows(spmv_matrix *h, const int32_t *rowptr, int64_t nrows, int64_
 }
 
 void free_packed(spmv_matrix *h) {
-    auto f = [](void *p) { if (p) cudaFree(p); };
+    auto f = [](void *p) { dev_free(p); };
     f(h->coo_rows); h->coo_rows = nullptr;
-    f(h->ell_col); h->ell_col = nullptr;
-    f(h->ell_d16); h->ell_d16 = nullptr;
-    f(h->ell_val); h->ell_val = nullptr;
+    f(h->ell_val); h->ell_val = nullptr;  // index arrays go with the values
+    h->ell_col = nullptr;
+    h->ell_d16 = nullptr;
     f(h->dia_ptr); h->dia_ptr = nullptr;
-    f(h->dia_off); h->dia_off = nullptr;
-    f(h->dia_mask); h->dia_mask = nullptr;
     f(h->dia_val); h->dia_val = nullptr;
+    h->dia_off = nullptr;
+    h->dia_mask = nullptr;
     h->dia_total = 0;
     h->ell_width = h->ell_pitch = 0;
     f(h->hyb_rows); h->hyb_rows = nullptr;
@@ -1498,8 +1520,8 @@ void free_packed(spmv_matrix *h) {
     f(h->bsr_col); h->bsr_col = nullptr;
     f(h->bsr_val); h->bsr_val = nullptr;
     f(h->sell_ptr); h->sell_ptr = nullptr;
-    f(h->sell_col); h->sell_col = nullptr;
     f(h->sell_val); h->sell_val = nullptr;
+    h->sell_col = nullptr;
     f(h->sell_perm); h->sell_perm = nullptr;
     h->sell_nslices = h->sell_slots = 0;
     h->bsr_r = 0;
@@ -1589,9 +1611,8 @@ int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, boo
     SPMV_TRY(dalloc(&h->dia_ptr, (size_t)nslices + 1));
     SPMV_TRY(exclusive_scan(count.p, h->dia_ptr, nslices + 1, s, &total));
     h->dia_total = total;
-    SPMV_TRY(dalloc(&h->dia_off, (size_t)total));
-    SPMV_TRY(dalloc(&h->dia_mask, (size_t)total * R));
-    SPMV_TRY(dalloc_bytes(&h->dia_val, sizeof(V) * (size_t)total * 32 * R));
+    SPMV_TRY(dalloc_slab({slab_bytes(&h->dia_val, sizeof(V) * (size_t)total * 32 * R), slab(&h->dia_off, (size_t)total),
+                          slab(&h->dia_mask, (size_t)total * R)}));
     auto fill = k_dia_slices<V, R, true>;
     shape(4 + sizeof(V), &nw, &smem);
     SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1633,12 +1654,11 @@ int pack_ell(spmv_matrix *h, int64_t width, cudaStream_t s) {
     else if (h->vt == SPMV_F32) SPMV_TRY(pack_dia<float>(h, width, index_bytes, s, &dia));
     else SPMV_TRY(pack_dia<__nv_bfloat16>(h, width, index_bytes, s, &dia));
     if (dia) return SPMV_OK;
-    SPMV_TRY(dalloc_bytes(&h->ell_val, vs * width * pitch));
     if (maxoff <= 32767) {
-        SPMV_TRY(dalloc(&h->ell_d16, (size_t)(width * pitch)));
+        SPMV_TRY(dalloc_slab({slab_bytes(&h->ell_val, vs * width * pitch), slab(&h->ell_d16, (size_t)(width * pitch))}));
         if (width > 0 && pitch > 0) SPMV_TRY(launch_ell_pack<int16_t>(h, width, pitch, h->ell_d16, s));
     } else {
-        SPMV_TRY(dalloc(&h->ell_col, (size_t)(width * pitch)));
+        SPMV_TRY(dalloc_slab({slab_bytes(&h->ell_val, vs * width * pitch), slab(&h->ell_col, (size_t)(width * pitch))}));
         if (width > 0 && pitch > 0) SPMV_TRY(launch_ell_pack<int>(h, width, pitch, h->ell_col, s));
     }
     return SPMV_OK;
@@ -1777,8 +1797,7 @@ int pack_sell(spmv_matrix *h, int kmax, bool grouped, cudaStream_t s) {
     SPMV_TRY(dalloc(&h->sell_perm, (size_t)std::max<int64_t>(m, 1)));
     if (m == 0) {
         SPMV_CUDA_TRY(cudaMemsetAsync(h->sell_ptr, 0, sizeof(int), s));
-        SPMV_TRY(dalloc(&h->sell_col, 1));
-        SPMV_TRY(dalloc_bytes(&h->sell_val, vs));
+        SPMV_TRY(dalloc_slab({slab_bytes(&h->sell_val, vs), slab(&h->sell_col, 1)}));
         h->sell_slots = 0;
         return SPMV_OK;
     }
@@ -1805,8 +1824,7 @@ int pack_sell(spmv_matrix *h, int kmax, bool grouped, cudaStream_t s) {
         return SPMV_ERR_UNSUPPORTED;
     }
     h->sell_slots = total;
-    SPMV_TRY(dalloc(&h->sell_col, (size_t)total));
-    SPMV_TRY(dalloc_bytes(&h->sell_val, vs * total));
+    SPMV_TRY(dalloc_slab({slab_bytes(&h->sell_val, vs * total), slab(&h->sell_col, (size_t)total)}));
     // work items (slice, first slot, column count <= kmax) and the partials
     // joining the items of one slice
     LongRows &L = h->lng;
@@ -1871,7 +1889,7 @@ int ensure_seg_scratch(spmv_matrix *h, int items, int kind, cudaStream_t s) {
     const int64_t nnz = kind != SEG_COO ? h->nnz : (h->cfg.format == SPMV_FMT_HYB ? h->hyb_nnz : h->nnz);
     const int C = 32 * items;
     const int64_t nchunks = (nnz + C - 1) / C;
-    auto f = [](void *p) { if (p) cudaFree(p); };
+    auto f = [](void *p) { dev_free(p); };
     f(g.meta0); f(g.meta1);
     free_partials(&g.part);
     g = SegScratch{};

@@ -39,6 +39,12 @@ inline cudaError_t dev_malloc_async(T **p, size_t bytes, cudaStream_t s) {
 }
 void entry_reset();
 
+// Frees what dev_malloc gave (null is fine).  The block may still be in use by
+// work already launched: it is handed out again only after a real cudaFree.
+// dev_free_waiting is that: it returns once the device's work is done.
+void dev_free(void *p);
+void dev_free_waiting(void *p);
+
 #define SPMV_CUDA_TRY(expr)                                       \
     do {                                                          \
         cudaError_t _e = (expr);                                  \
@@ -319,12 +325,13 @@ struct spmv_matrix {
     int sm_count = 0;
     // CSR (always present: the base every other format is packed from)
     int32_t *rowptr = nullptr;
-    int32_t *colidx = nullptr;
+    int32_t *colidx = nullptr;  // in one block behind vals
     void *vals = nullptr;
     // COO row array (COO format; column and value arrays alias the CSR ones)
     int32_t *coo_rows = nullptr;
     // ELL (also the ELL part of HYB)
     int64_t ell_width = 0, ell_pitch = 0;
+    // (index arrays of a format sit in one block behind its values)
     int32_t *ell_col = nullptr;   // int32 columns, padding -1 ...
     int16_t *ell_d16 = nullptr;   // ... or 16-bit column - row, padding INT16_MIN
     void *ell_val = nullptr;
@@ -396,7 +403,7 @@ int build_long_rows(spmv_matrix *h, const int32_t *rowptr, int64_t nrows, int64_
 // row panels (convert.cu): bounds check of every triplet; panel row bounds
 // (multiples of 4 rows, at most `limit` triplets each); stable copy of the
 // triplets of rows [r0, r1) with rows shifted by -r0 (device buffers the
-// caller frees with cudaFree)
+// caller frees with dev_free)
 int check_triplet_bounds(const int32_t *d_rows, const int32_t *d_cols, int64_t nnz, int64_t m, int64_t n,
                          cudaStream_t s);
 int plan_panels(const int32_t *d_rows, int64_t nnz, int64_t m, int64_t limit, cudaStream_t s,

@@ -198,7 +198,7 @@ int selector_load_slot(int slot, const float *h_blob, int64_t count) {
             return SPMV_ERR_CUDA;
         }
         std::lock_guard<std::mutex> lk(g_sel_mu);
-        if (sel->d_w) cudaFree(sel->d_w);
+        dev_free(sel->d_w);
         *sel = Selector{};
         return SPMV_OK;
     }
@@ -236,7 +236,7 @@ int selector_load_slot(int slot, const float *h_blob, int64_t count) {
         return SPMV_ERR_CUDA;
     }
     std::lock_guard<std::mutex> lk(g_sel_mu);
-    if (sel->d_w) cudaFree(sel->d_w);
+    dev_free(sel->d_w);
     *sel = Selector{};
     // device layout: network weights, then (version 2) the time head
     std::vector<float> w(h_blob + 5, h_blob + 5 + nw1);
