@@ -728,7 +728,7 @@ __device__ __forceinline__ void ell_code(int16_t *p, int c, int64_t r) {
 // 101^3, fp64, 216 us, 156 now (its bytes at the HBM rate: 98), bound by
 // load latency at the 20 warps per SM that the staging leaves room for.
 // One padding word per 32 spreads rows of one length over the banks.
-constexpr int ELL_PACK_CAP = 4608, ELL_PACK_SMEM = 96 * 1024;
+constexpr int ELL_PACK_CAP = 4608, ELL_PACK_SMEM = 96 * 1024, DIA_PACK_CAP = 20480;
 __host__ __device__ inline size_t ell_pack_words(int cap) { return (size_t)cap + cap / 32 + 1; }
 
 template <typename V, typename CI>
@@ -774,92 +774,79 @@ __global__ void __launch_bounds__(128) k_ell_pack(const int *__restrict__ rowptr
 // Diagonals of a slice (32 R rows, of each row its first `width` entries): a
 // merge of the rows' ascending offsets, one step per distinct offset.  Without
 // FILL the steps are counted (given up past `most`), with FILL each step
-// writes its offset, row masks and values.  One warp per slice, every
-// step_s-th slice; the slice's columns and values are staged as in k_ell_pack.
+// writes its offset, row masks and values.  A block of R warps takes a slice
+// (warp w the rows 32 w .. 32 w + 31, a row per lane), every step_s-th slice;
+// the slice's columns and values are staged as in k_ell_pack, at most cap.
 template <typename V, int R, bool FILL>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(32 * R)
 k_dia_slices(const int *__restrict__ rowptr, const int *__restrict__ colidx, const V *__restrict__ vals, int64_t m,
              int64_t width, int64_t nslices, int64_t step_s, int most, int cap, const int *__restrict__ ptr, int *count,
              unsigned long long *sums, int *off, uint32_t *mask, V *val) {
     extern __shared__ __align__(16) unsigned char pack_smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const size_t words = ell_pack_words(cap);
-    V *sv = reinterpret_cast<V *>(pack_smem) + warp * words;
-    int *sc = FILL ? reinterpret_cast<int *>(pack_smem + (sizeof(V) * words * nw + 15) / 16 * 16) + warp * words
-                   : reinterpret_cast<int *>(pack_smem) + warp * words;
+    __shared__ int s_min[2][R];
+    __shared__ unsigned s_entries;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    int *sc = reinterpret_cast<int *>(pack_smem);
+    V *sv = reinterpret_cast<V *>(pack_smem + (4 * ell_pack_words(cap) + 15) / 16 * 16);
+    if (!FILL && tid == 0) s_entries = 0;
     unsigned diags = 0, entries = 0;
-    for (int64_t sl = ((int64_t)blockIdx.x * nw + warp) * step_s; sl < nslices; sl += (int64_t)gridDim.x * nw * step_s) {
-        int p[R], e[R], d[R];
-        int64_t row[R];
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-            row[i] = sl * (32 * R) + 32 * i + lane;
-            p[i] = __ldg(rowptr + (row[i] < m ? row[i] : m));
-            e[i] = __ldg(rowptr + (row[i] + 1 < m ? row[i] + 1 : m));
-        }
-        const int w0 = __shfl_sync(FULL, p[0], 0), w1 = __shfl_sync(FULL, e[R - 1], 31);
+    for (int64_t sl = (int64_t)blockIdx.x * step_s; sl < nslices; sl += (int64_t)gridDim.x * step_s) {
+        const int64_t first = sl * (32 * R), row = first + tid, end = first + 32 * R < m ? first + 32 * R : m;
+        const int w0 = __ldg(rowptr + first), w1 = __ldg(rowptr + end);
+        int p = __ldg(rowptr + (row < m ? row : m)), e = __ldg(rowptr + (row + 1 < m ? row + 1 : m));
         const bool staged = w1 - w0 <= cap;
-        __syncwarp();
+        __syncthreads();  // the previous slice's staging is read
         if (staged) {
 #pragma unroll 8
-            for (int o = lane; o < w1 - w0; o += 32) {
+            for (int o = tid; o < w1 - w0; o += 32 * R) {
                 sc[o + (o >> 5)] = __ldg(colidx + w0 + o);
                 if (FILL) sv[o + (o >> 5)] = vals[w0 + o];
             }
         }
-        __syncwarp();
+        __syncthreads();
         auto col = [&](int k) -> int { return staged ? sc[(k - w0) + ((k - w0) >> 5)] : __ldg(colidx + k); };
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-            if (e[i] - p[i] > width) e[i] = p[i] + (int)width;
-            entries += e[i] - p[i];
-            d[i] = p[i] < e[i] ? (int)(col(p[i]) - row[i]) : INT_MAX;
-        }
+        if (e - p > width) e = p + (int)width;
+        entries += e - p;
+        int d = p < e ? (int)(col(p) - row) : INT_MAX;
         int64_t at = FILL ? __ldg(ptr + sl) : 0;
         int n = 0;
-        for (;;) {
-            int lo = d[0];
+        for (;; ++n) {
+            int lo = __reduce_min_sync(FULL, d);
+            if (R > 1) {  // over the block's warps; two sets, so one barrier a step
+                if (lane == 0) s_min[n & 1][w] = lo;
+                __syncthreads();
 #pragma unroll
-            for (int i = 1; i < R; ++i) lo = min(lo, d[i]);
-            lo = __reduce_min_sync(FULL, lo);
-            if (lo == INT_MAX || (!FILL && n == most)) break;
-            V v[R];
-            uint32_t w[R];
-#pragma unroll
-            for (int i = 0; i < R; ++i) {
-                const bool hit = d[i] == lo;
-                if (FILL) {
-                    w[i] = __ballot_sync(FULL, hit);
-                    v[i] = V(0.0f);
-                    if (hit) v[i] = staged ? sv[(p[i] - w0) + ((p[i] - w0) >> 5)] : vals[p[i]];
-                }
-                if (hit) {
-                    ++p[i];
-                    d[i] = p[i] < e[i] ? (int)(col(p[i]) - row[i]) : INT_MAX;
-                }
+                for (int i = 0; i < R; ++i) lo = min(lo, s_min[n & 1][i]);
             }
+            if (lo == INT_MAX || (!FILL && n == most)) break;
+            const bool hit = d == lo;
             if (FILL) {
-                if (lane == 0) {
-                    off[at] = lo;
-#pragma unroll
-                    for (int i = 0; i < R; ++i) mask[at * R + i] = w[i];
-                }
-#pragma unroll
-                for (int i = 0; i < R; ++i) val[(at * 32 + lane) * R + i] = v[i];
+                const uint32_t bits = __ballot_sync(FULL, hit);
+                V v = V(0.0f);
+                if (hit) v = staged ? sv[(p - w0) + ((p - w0) >> 5)] : vals[p];
+                if (tid == 0) off[at] = lo;
+                if (lane == 0) mask[at * R + w] = bits;
+                val[(at * 32 + lane) * R + w] = v;
                 ++at;
             }
-            ++n;
+            if (hit) {
+                ++p;
+                d = p < e ? (int)(col(p) - row) : INT_MAX;
+            }
         }
         if (!FILL) {
-            if (lane == 0 && count) count[sl] = n;
+            if (tid == 0 && count) count[sl] = n;
             diags += n;
         }
     }
     if (!FILL) {
+        __syncthreads();
         entries = __reduce_add_sync(FULL, entries);
-        if (lane == 0) {
+        if (lane == 0) atomicAdd(&s_entries, entries);
+        __syncthreads();
+        if (tid == 0) {
             atomicAdd(sums, (unsigned long long)diags);
-            atomicAdd(sums + 1, (unsigned long long)entries);
+            atomicAdd(sums + 1, (unsigned long long)s_entries);
         }
     }
 }
@@ -1568,26 +1555,25 @@ int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, boo
     *done = false;
     const int64_t m = h->m, nslices = (m + 32 * R - 1) / (32 * R);
     if (width == 0 || h->nnz < (1 << 20)) return SPMV_OK;
-    const int cap = (int)std::min<int64_t>(ELL_PACK_CAP, 32 * R * width);
-    auto shape = [&](size_t entry_bytes, int *nw, size_t *smem) {
-        const size_t per_warp = ell_pack_words(cap) * entry_bytes;
-        *nw = (int)std::max<size_t>(1, std::min<size_t>(4, ELL_PACK_SMEM / per_warp));
-        *smem = per_warp * *nw + 16;
+    // staging for a slice's entries: read in place, long rows fall out of L1
+    // between steps (band of half-width 32, bf16, 300,000 rows: 198 us a count and
+    // 335 a fill with a warp per slice in place, 29 and 147 staged, a warp per 32 rows)
+    const int cap = (int)std::min<int64_t>(DIA_PACK_CAP, 32 * R * width);
+    auto smem_of = [&](bool values) {
+        return (4 * ell_pack_words(cap) + 15) / 16 * 16 + (values ? sizeof(V) * ell_pack_words(cap) : 0);
     };
-    int nw;
-    size_t smem;
     Tmp<unsigned long long> sums;
     Tmp<int> count;
     SPMV_TRY(sums.alloc(2, s));
     auto count_kernel = k_dia_slices<V, R, false>;
-    shape(4, &nw, &smem);
-    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem_of(false)));
     // the diagonals of `slices` slices (one in step_s) and the entries on them
     auto counted = [&](int64_t step_s, int *out, bool *worth) -> int {
         const int64_t slices = (nslices + step_s - 1) / step_s;
         unsigned long long hs[2];
         SPMV_CUDA_TRY(cudaMemsetAsync(sums.p, 0, sizeof(hs), s));
-        count_kernel<<<grid1d(slices, nw, 1 << 20), 32 * nw, smem, s>>>(
+        count_kernel<<<grid1d(slices, 1, 152 * 32), 32 * R, smem_of(false), s>>>(
             h->rowptr, h->colidx, (const V *)h->vals, m, width, nslices, step_s, (int)std::min<int64_t>(4 * width + 16, 1 << 20),
             cap, nullptr, out, sums.p, nullptr, nullptr, nullptr);
         SPMV_CUDA_TRY(cudaGetLastError());
@@ -1614,9 +1600,9 @@ int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, boo
     SPMV_TRY(dalloc_slab({slab_bytes(&h->dia_val, sizeof(V) * (size_t)total * 32 * R), slab(&h->dia_off, (size_t)total),
                           slab(&h->dia_mask, (size_t)total * R)}));
     auto fill = k_dia_slices<V, R, true>;
-    shape(4 + sizeof(V), &nw, &smem);
-    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    fill<<<grid1d(nslices, nw, 1 << 20), 32 * nw, smem, s>>>(h->rowptr, h->colidx, (const V *)h->vals, m, width, nslices, 1,
+    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)fill, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem_of(true)));
+    fill<<<grid1d(nslices, 1, 1 << 30), 32 * R, smem_of(true), s>>>(h->rowptr, h->colidx, (const V *)h->vals, m, width, nslices, 1,
                                                              INT_MAX, cap, h->dia_ptr, nullptr, nullptr, h->dia_off,
                                                              h->dia_mask, (V *)h->dia_val);
     SPMV_CUDA_TRY(cudaGetLastError());
