@@ -14,11 +14,29 @@ namespace spmv {
 // occupancy-limited resident blocks per SM for (kernel, block size); cached
 int resident_blocks(const void *kernel, int threads);
 
-// grid of at most one full wave of resident blocks (grid-stride kernels)
-inline int wave_grid(const void *kernel, int threads, int64_t needed_blocks, int sm_count) {
-    const int64_t cap = (int64_t)resident_blocks(kernel, threads) * sm_count;
+// Grid of at most `waves` times the resident blocks (grid-stride kernels).
+// One wave is best where every warp's share takes the same time: blocks start
+// once and their loads follow each other without a gap.  Where shares differ
+// (gathers that miss at random, uneven rows) a fixed share leaves the chip
+// waiting for its slowest warps, and blocks handed out as others end balance it
+// (from three waves of them on: Poisson(40) 200,000 rows SELL fp32, 1.3 waves, 30.6
+// us in one wave, 35.6 with all blocks).
+constexpr int64_t ONE_WAVE = 1, ALL_BLOCKS = int64_t(1) << 30;
+inline int wave_grid(const void *kernel, int threads, int64_t needed_blocks, int sm_count, int64_t waves = ONE_WAVE) {
+    int64_t cap = (int64_t)resident_blocks(kernel, threads) * sm_count;
+    if (needed_blocks >= 3 * cap) cap = std::min<int64_t>(cap * waves, 0x7fffffff);
     int64_t g = needed_blocks < cap ? needed_blocks : cap;
     return (int)(g < 1 ? 1 : g);
+}
+
+// Scattered columns (under a quarter of consecutive entries in consecutive
+// columns, the layouts' rule) with rows of eight entries and more: all blocks
+// at once for ELL and SELL.  One wave / all blocks, us, SELL: Poisson(16) 2^20
+// rows fp32 69.4 / 65.7, fp64 74.9 / 71.3, R-MAT scale 20 fp32 60.8 / 50.5, fp64
+// 69.5 / 61.7; ELL part of HYB, Poisson(16) fp64 88.3 / 82.1; but Poisson(4) SELL
+// 24.2 / 24.8 and the 27-point stencil fp32 80.3 / 87.9.
+inline int64_t row_waves(const spmv_matrix *h) {
+    return h->contig < 0.25 && h->nnz >= 8 * h->m ? ALL_BLOCKS : ONE_WAVE;
 }
 
 #define SPMV_LAUNCH_CHECK()                                      \
@@ -134,12 +152,12 @@ int launch_ell_ci(const spmv_matrix *h, const CI *cols, int64_t width, T alpha, 
         auto kern = k_ell2<V, T, U, RC, CI>;
         SPMV_TRY(apply_carveout((const void *)kern, h->cfg.carveout));
         const int64_t pairs = (h->m + 1) / 2;
-        const int grid = wave_grid((const void *)kern, tpb, (pairs + tpb - 1) / tpb, h->sm_count);
+        const int grid = wave_grid((const void *)kern, tpb, (pairs + tpb - 1) / tpb, h->sm_count, row_waves(h));
         kern<<<grid, tpb, 0, s>>>(h->m, width, h->ell_pitch, cols, (const V *)h->ell_val, x, y, alpha, beta);
     } else {
         auto kern = k_ell<V, T, U, RC, CI>;
         SPMV_TRY(apply_carveout((const void *)kern, h->cfg.carveout));
-        const int grid = wave_grid((const void *)kern, tpb, (h->m + tpb - 1) / tpb, h->sm_count);
+        const int grid = wave_grid((const void *)kern, tpb, (h->m + tpb - 1) / tpb, h->sm_count, row_waves(h));
         kern<<<grid, tpb, 0, s>>>(h->m, width, h->ell_pitch, cols, (const V *)h->ell_val, x, y, alpha, beta);
     }
     SPMV_LAUNCH_CHECK();
@@ -236,7 +254,7 @@ int launch_sell_g(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, cudaS
     const int64_t wpb = tpb / 32;
     const int64_t empty_rows = h->m - 32 * L.nrows > 0 ? h->m - 32 * L.nrows : 0;
     const int64_t need = std::max((L.nseg + wpb - 1) / wpb, (empty_rows + tpb - 1) / tpb);
-    const int grid = wave_grid((const void *)kern, tpb, need, h->sm_count);
+    const int grid = wave_grid((const void *)kern, tpb, need, h->sm_count, row_waves(h));
     kern<<<grid, tpb, 0, s>>>(h->m, L.nseg, L.nrows, L.seg_row, L.seg_begin, L.seg_end, L.seg_c0, L.seg_c1, h->sell_col,
                               (const V *)h->sell_val, h->sell_perm, x, y, alpha, beta, PartialsT<T>::of(L.part));
     SPMV_LAUNCH_CHECK();
@@ -280,7 +298,10 @@ int launch_coo(const spmv_matrix *h, int64_t nnz, const int *rows, const int *co
     SPMV_TRY(apply_carveout((const void *)kern, h->cfg.carveout));
     const int64_t chunks = (nnz + 32 * ITEMS - 1) / (32 * ITEMS);
     const int64_t wpb = tpb / 32;
-    const int grid = wave_grid((const void *)kern, tpb, (chunks + wpb - 1) / wpb, h->sm_count);
+    // uneven rows: runs of equal rows differ from chunk to chunk (R-MAT scale 20, one / four waves: fp32 98.6 /
+    // 90.1 us, fp64 122.0 / 109.4; Poisson(16) fp32 79.9 / 83.4)
+    const int grid = wave_grid((const void *)kern, tpb, (chunks + wpb - 1) / wpb, h->sm_count,
+                               csr_uneven(h, 1) ? 4 : ONE_WAVE);
     kern<<<grid, tpb, 0, s>>>(nnz, h->m, rows, cols, vals, x, y, alpha, beta, h->seg.meta0, h->seg.meta1,
                               PartialsT<T>::of(h->seg.part));
     SPMV_LAUNCH_CHECK();
