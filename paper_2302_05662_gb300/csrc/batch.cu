@@ -1,14 +1,24 @@
 // Batched SpMV: hundreds of uneven matrices in one persistent launch.
 //
-// Each matrix contributes work items for one warp each, in the format its
-// handle holds: ELL (groups of 32 rows, a row per lane), SELL (the handle's
-// work items, plus groups of 32 of its empty rows), or otherwise CSR --
-// chunks of 32*ITEMS nonzeros (split mode, for power-law or very short rows)
-// or groups of 32 rows with a per-matrix number of lanes per row (vector
-// mode).  A grid of
-// resident thread blocks pulls items from one atomic counter, so small and
-// large matrices share the GPU without a launch per matrix.  The counter
-// reset and the kernel are captured once in a CUDA graph and replayed.  An
+// Each matrix is cut into units of one pass of a warp, in the format its
+// handle holds: ELL (32 rows, a row per lane, or a slice of diagonals), SELL
+// (the handle's work items, plus groups of 32 of its empty rows), BSR (as many
+// block rows as a warp holds), COO chunks, or otherwise CSR -- chunks of
+// 32*ITEMS nonzeros (split mode, for power-law or very short rows) or as many
+// rows as a warp holds with a per-matrix number of lanes per row (vector
+// mode).  An item is one to four units of a matrix, about 1024 entries
+// whatever the format, so that no item is much longer than another (four
+// units of 32 rows each held 500 entries of one matrix and 16,000 of the
+// next, the last of which ended long after the others).  A grid of resident thread blocks
+// pulls items from one atomic counter, so small and large matrices share the
+// GPU without a launch per matrix; a map made once gives an item's matrix and
+// first unit, and the warp that draws last resets the counter.  96 mixed fp32
+// matrices of 1000 to 200,000 rows (99.5M entries): 357 us before (items of four
+// units, a binary search per item, a counter reset per launch), 264 now; it
+// waits on its loads (x gathers from L2 for the 31M scattered entries).  Fewer
+// or more warps in flight lose: 72 or 80 registers 334 and 324 us against 292
+// with 64, 4 entries a lane 337 against 277.  The
+// kernel is captured once in a CUDA graph and replayed.  An
 // autotuner times the per-matrix mode and the batch-wide chunk and block
 // sizes (the paper's compile-time parameters of Section 4, chosen per
 // matrix by measurement instead of by a model).
@@ -20,7 +30,7 @@
 
 struct spmv_batch {
     int count = 0, vt = SPMV_F64, items = 8, tpb = 256, sm_count = 0;
-    int group = 4;  // work units (chunks, row groups, SELL items) per batch item
+    int group = 4;  // stored entries per batch item, in steps of 256
     std::vector<spmv_handle> hs;
     std::vector<double> alpha, beta;
     std::vector<const void *> x;
@@ -28,7 +38,7 @@ struct spmv_batch {
     std::vector<int> modes;  // 0 split, else threads per row
     // device state
     void *d_mats = nullptr;
-    int64_t *d_item_off = nullptr;
+    int2 *d_items = nullptr;  // matrix and first unit of each item
     int64_t total_items = 0;
     std::vector<int32_t *> metas;
     spmv::Partials part;
@@ -50,7 +60,8 @@ struct BatchMat {
     double alpha, beta;
     int64_t m, nnz;
     int64_t part_off;  // first chunk of this matrix in the batch partials
-    int64_t units;     // work units of this matrix (batch items take `group` of them)
+    int64_t units;     // work units of this matrix
+    int group;         // ... of which an item takes this many
     const int *meta0;  // split: first row starting at or after each chunk's first entry;
                        // COO: first chunk of each chunk's head row
     const int *meta1;  // COO: last chunk of each chunk's tail row
@@ -59,7 +70,7 @@ struct BatchMat {
     const int *bsr_rowptr, *bsr_col;
     const void *bsr_val;
     int64_t bsr_mb, n;
-    int bsr_r, pad3;
+    int bsr_r, bsr_s;  // ... and the blocks of a block row taken at once
     int mode;          // CSR: 0 split, -2 COO chunks, else lanes per row
     int fmt;           // the handle's format: SPMV_FMT_ELL, SPMV_FMT_SELL, or CSR (any other)
     // ELL: column-major arrays, int32 columns or 16-bit offsets
@@ -86,18 +97,37 @@ struct BatchMat {
 };
 
 // mode of a COO handle run as COO chunks (its own row indices), of a BSR
-// handle run as BSR block rows (32 / r block rows per item, r lanes each)
+// handle run as BSR block rows (r bsr_s lanes each)
 constexpr int BATCH_COO = -SPMV_FMT_COO;
 constexpr int BATCH_BSR = -SPMV_FMT_BSR;
 
-// work items of one matrix: CSR split or COO chunks, or 32-row groups, ELL
-// 32-row groups, SELL items plus 32-row groups of its empty rows
+// work units of one matrix: CSR split or COO chunks, the CSR rows or BSR block
+// rows of one pass of a warp, ELL 32-row groups or slices of diagonals, SELL
+// items plus 32-row groups of its empty rows
 int64_t batch_items(const BatchMat &M, int C) {
     if (M.fmt == SPMV_FMT_ELL && M.dia_val) return (M.m + 32 * M.dia_r - 1) / (32 * M.dia_r);
     if (M.fmt == SPMV_FMT_ELL) return (M.m + 31) / 32;
     if (M.fmt == SPMV_FMT_SELL) return M.nitems + (std::max<int64_t>(0, M.m - 32 * M.s_zero) + 31) / 32;
-    if (M.fmt == SPMV_FMT_BSR) return (M.bsr_mb + 32 / M.bsr_r - 1) / (32 / M.bsr_r);
-    return M.mode == 0 || M.mode == BATCH_COO ? (M.nnz + C - 1) / C : (M.m + 31) / 32;
+    if (M.fmt == SPMV_FMT_BSR) return (M.bsr_mb * M.bsr_r * M.bsr_s + 31) / 32;
+    return M.mode == 0 || M.mode == BATCH_COO ? (M.nnz + C - 1) / C : (M.m * M.mode + 31) / 32;
+}
+
+// units of a matrix in one item: about 256 `steps` entries, in at most four
+// units (a warp's units follow each other: with eight, 14 block-diagonal
+// matrices of 1.2M entries in all took 46 us instead of 24)
+int item_units(const BatchMat &M, int steps) {
+    const double per_unit = (double)std::max<int64_t>(M.nnz, 1) / (double)std::max<int64_t>(M.units, 1);
+    return (int)std::max(1.0, std::min(4.0, std::floor(steps * 256.0 / per_unit + 0.5)));
+}
+
+// blocks of a block row taken at once: a quarter of a mean block row's, at
+// most 8 (one at a time, a 129-wide band's block row was a chain of 16 loads
+// on a lane; ten such matrices, 42M entries: 90 us / 71 with the x blocks)
+int bsr_lanes(const spmv_matrix *h) {
+    const double mean = h->bsr_mb > 0 ? (double)h->bsr_blocks / (double)h->bsr_mb : 0.0;
+    int s = 1;
+    while (s < 8 && 2.0 * s <= mean / 4.0) s *= 2;
+    return s;
 }
 
 // chunk metadata of a split or COO matrix for chunks of C entries, in one
@@ -126,6 +156,7 @@ void describe_format(const spmv_matrix *h, BatchMat &M) {
         M.bsr_val = h->bsr_val;
         M.bsr_mb = h->bsr_mb;
         M.bsr_r = h->bsr_r;
+        M.bsr_s = bsr_lanes(h);
     }
     M.n = h->n;
     if (h->cfg.format == SPMV_FMT_ELL && (h->ell_col || h->ell_d16 || h->dia_val)) {
@@ -161,7 +192,6 @@ void describe_format(const spmv_matrix *h, BatchMat &M) {
     }
 }
 
-// register budget: 16 items per lane, or fp64 sums, need more than 64
 // vector mode with one or two lanes per row takes 8-entry load groups once
 // a lane's part of a mean row holds 16 or more entries (the single-matrix
 // default rule)
@@ -170,25 +200,27 @@ int wide_groups(const spmv_matrix *h, int mode) {
     return mode >= 1 && mode <= 2 && mean / mode >= 16.0 ? 1 : 0;
 }
 
+// register budget: 16 items per lane, or fp64 sums, need more than 64
 template <typename V, typename T, int ITEMS>
 __global__ void __launch_bounds__(512) __maxnreg__(ITEMS >= 16 ? 128 : (sizeof(T) == 8 ? 96 : 64))
-k_batch(const BatchMat *__restrict__ mats, int count, const int64_t *__restrict__ item_off, int64_t total,
-        int group, unsigned long long *counter, const PartialsT<T> P) {
+k_batch(const BatchMat *__restrict__ mats, const int2 *__restrict__ items, int64_t total,
+        unsigned long long *counter, const PartialsT<T> P) {
     __shared__ MergeSmem<ITEMS> s_merge[16];  // split chunks: one per warp
     const int lane = threadIdx.x & 31;
     for (;;) {
         unsigned long long item = 0;
         if (lane == 0) item = atomicAdd(counter, 1ull);
         item = __shfl_sync(0xffffffffu, item, 0);
-        if (item >= (unsigned long long)total) break;
-        int lo = 0, hi = count - 1;  // matrix owning the item
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if ((unsigned long long)__ldg(item_off + mid) <= item) lo = mid; else hi = mid - 1;
+        if (item >= (unsigned long long)total) {
+            // each warp draws past the end once: the last one to do so resets the counter
+            const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+            if (lane == 0 && item == (unsigned long long)total + warps - 1) *counter = 0;
+            break;
         }
-        const BatchMat &M = mats[lo];  // fields read where a branch needs them
-        const int64_t u0 = ((int64_t)item - __ldg(item_off + lo)) * group;
-        const int64_t u1 = u0 + group < M.units ? u0 + group : M.units;
+        const int2 at = __ldg(items + item);  // matrix and first unit
+        const BatchMat &M = mats[at.x];  // fields read where a branch needs them
+        const int64_t u0 = at.y;
+        const int64_t u1 = u0 + M.group < M.units ? u0 + M.group : M.units;
         const Epi<T> ep((T)M.alpha, (T)M.beta);
         const V *vals = (const V *)M.vals;
         const T *x = (const T *)M.x;
@@ -220,10 +252,10 @@ k_batch(const BatchMat *__restrict__ mats, int count, const int64_t *__restrict_
         } else if (M.fmt == SPMV_FMT_BSR) {  // 32 / r block rows, r lanes per block row
             const int big = 0x7fffffff;
             if (M.bsr_r == 4)
-                bsr_rows<V, T, 4, 1>(local * 8, M.bsr_mb, M.m, M.n, M.bsr_rowptr, M.bsr_col, (const V *)M.bsr_val, x,
+                bsr_rows<V, T, 4>(local * (8 / M.bsr_s), M.bsr_s, M.bsr_mb, M.m, M.n, M.bsr_rowptr, M.bsr_col, (const V *)M.bsr_val, x,
                                      y, ep, big);
             else
-                bsr_rows<V, T, 2, 1>(local * 16, M.bsr_mb, M.m, M.n, M.bsr_rowptr, M.bsr_col, (const V *)M.bsr_val,
+                bsr_rows<V, T, 2>(local * (16 / M.bsr_s), M.bsr_s, M.bsr_mb, M.m, M.n, M.bsr_rowptr, M.bsr_col, (const V *)M.bsr_val,
                                      x, y, ep, big);
         } else if (M.mode == 0 || M.mode == BATCH_COO) {
             PartialsT<T> Pm = P;
@@ -239,61 +271,77 @@ k_batch(const BatchMat *__restrict__ mats, int count, const int64_t *__restrict_
                                              __ldg(M.meta0 + local), __ldg(M.meta0 + local + 1), Pm,
                                              s_merge[threadIdx.x >> 5]);
         } else {
-            const int64_t base = local * 32;
             const int big = 0x7fffffff;
+            const int64_t base = local * (32 / M.mode);
             switch (M.mode) {
             case 1:
                 if (M.wide) csr_vector_rows<V, T, 1, 2, 8>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big);
                 else csr_vector_rows<V, T, 1, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big);
                 break;
             case 2:
-                if (M.wide) csr_vector_rows<V, T, 2, 2, 8>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big);
-                else csr_vector_rows<V, T, 2, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big);
+                if (M.wide) csr_vector_rows<V, T, 2, 2, 8>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big, 1);
+                else csr_vector_rows<V, T, 2, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big, 1);
                 break;
-            case 4: csr_vector_rows<V, T, 4, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big); break;
-            case 8: csr_vector_rows<V, T, 8, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big); break;
-            case 16: csr_vector_rows<V, T, 16, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big); break;
-            default: csr_vector_rows<V, T, 32, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big); break;
+            case 4: csr_vector_rows<V, T, 4, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big, 1); break;
+            case 8: csr_vector_rows<V, T, 8, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big, 1); break;
+            case 16: csr_vector_rows<V, T, 16, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big, 1); break;
+            default: csr_vector_rows<V, T, 32, 2>(base, M.m, M.rowptr, M.colidx, vals, x, y, ep, big, 1); break;
             }
         }
         }
     }
 }
 
+// items[i] = matrix and first unit of item i (items of matrix k are [off[k], off[k+1]))
+__global__ void k_batch_items(const BatchMat *mats, const int64_t *off, int count, int64_t total, int2 *items) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+        int lo = 0, hi = count - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (off[mid] <= i) lo = mid; else hi = mid - 1;
+        }
+        items[i] = make_int2(lo, (int)((i - off[lo]) * mats[lo].group));
+    }
+}
+
+int fill_items(const BatchMat *mats, const int64_t *off, int count, int64_t total, int2 *items, cudaStream_t s) {
+    if (total == 0) return SPMV_OK;
+    k_batch_items<<<(unsigned)std::min<int64_t>((total + 255) / 256, 4096), 256, 0, s>>>(mats, off, count, total, items);
+    SPMV_CUDA_TRY(cudaGetLastError());
+    return SPMV_OK;
+}
+
 template <typename V, typename T, int ITEMS>
-int launch_batch_t(const spmv_batch *b, const BatchMat *mats, int count, const int64_t *item_off, int64_t total,
-                   cudaStream_t s) {
+int launch_batch_t(const spmv_batch *b, const BatchMat *mats, const int2 *items, int64_t total, cudaStream_t s) {
     auto kern = k_batch<V, T, ITEMS>;
     const int per_sm = resident_blocks((const void *)kern, b->tpb);
     const int64_t need = (total + b->tpb / 32 - 1) / (b->tpb / 32);
     const int64_t cap = (int64_t)per_sm * b->sm_count;
     const int grid = (int)std::max<int64_t>(1, std::min(need, cap));
-    kern<<<grid, b->tpb, 0, s>>>(mats, count, item_off, total, b->group, b->d_counter, PartialsT<T>::of(b->part));
+    kern<<<grid, b->tpb, 0, s>>>(mats, items, total, b->d_counter, PartialsT<T>::of(b->part));
     SPMV_CUDA_TRY(cudaGetLastError());
     return SPMV_OK;
 }
 
 template <int VT>
-int launch_batch_vt(const spmv_batch *b, const BatchMat *mats, int count, const int64_t *item_off, int64_t total,
-                    cudaStream_t s) {
+int launch_batch_vt(const spmv_batch *b, const BatchMat *mats, const int2 *items, int64_t total, cudaStream_t s) {
     using V = typename VT_<VT>::V;
     using T = typename VT_<VT>::T;
     switch (b->items) {
-    case 4: return launch_batch_t<V, T, 4>(b, mats, count, item_off, total, s);
-    case 16: return launch_batch_t<V, T, 16>(b, mats, count, item_off, total, s);
-    default: return launch_batch_t<V, T, 8>(b, mats, count, item_off, total, s);
+    case 4: return launch_batch_t<V, T, 4>(b, mats, items, total, s);
+    case 16: return launch_batch_t<V, T, 16>(b, mats, items, total, s);
+    default: return launch_batch_t<V, T, 8>(b, mats, items, total, s);
     }
 }
 
-// counter reset + one persistent kernel over `count` descriptors
-int launch_batch(const spmv_batch *b, const BatchMat *mats, int count, const int64_t *item_off, int64_t total,
-                 cudaStream_t s) {
-    SPMV_CUDA_TRY(cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned long long), s));
+// one persistent kernel over the items
+int launch_batch(const spmv_batch *b, const BatchMat *mats, const int2 *items, int64_t total, cudaStream_t s) {
     if (total == 0) return SPMV_OK;
     switch (b->vt) {
-    case SPMV_F64: return launch_batch_vt<SPMV_F64>(b, mats, count, item_off, total, s);
-    case SPMV_F32: return launch_batch_vt<SPMV_F32>(b, mats, count, item_off, total, s);
-    default: return launch_batch_vt<SPMV_BF16>(b, mats, count, item_off, total, s);
+    case SPMV_F64: return launch_batch_vt<SPMV_F64>(b, mats, items, total, s);
+    case SPMV_F32: return launch_batch_vt<SPMV_F32>(b, mats, items, total, s);
+    default: return launch_batch_vt<SPMV_BF16>(b, mats, items, total, s);
     }
 }
 
@@ -312,9 +360,9 @@ void free_device(spmv_batch *b) {
     b->exec = nullptr;
     b->graph = nullptr;
     dev_free(b->d_mats);
-    dev_free(b->d_item_off);
+    dev_free(b->d_items);
     b->d_mats = nullptr;
-    b->d_item_off = nullptr;
+    b->d_items = nullptr;
     for (int32_t *p : b->metas)
         dev_free(p);
     b->metas.clear();
@@ -360,19 +408,26 @@ int build(spmv_batch *b, cudaStream_t s) {
             chunks_total += nch;
         }
         M.units = batch_items(M, C);
-        off[i + 1] = off[i] + (M.units + b->group - 1) / b->group;
+        M.group = item_units(M, b->group);
+        off[i + 1] = off[i] + (M.units + M.group - 1) / M.group;
     }
     b->total_items = off[b->count];
     SPMV_TRY(alloc_partials(&b->part, chunks_total, 1, b->vt, s));
     SPMV_CUDA_TRY(dev_malloc(&b->d_mats, sizeof(BatchMat) * std::max(1, b->count)));
-    SPMV_CUDA_TRY(dev_malloc((void **)&b->d_item_off, sizeof(int64_t) * (b->count + 1)));
-    SPMV_CUDA_TRY(cudaMemcpyAsync(b->d_mats, mats.data(), sizeof(BatchMat) * b->count, cudaMemcpyHostToDevice, s));
-    SPMV_CUDA_TRY(cudaMemcpyAsync(b->d_item_off, off.data(), sizeof(int64_t) * (b->count + 1),
-                                  cudaMemcpyHostToDevice, s));
+    SPMV_CUDA_TRY(dev_malloc((void **)&b->d_items, sizeof(int2) * (size_t)std::max<int64_t>(1, b->total_items)));
+    int64_t *d_off = nullptr;
+    SPMV_CUDA_TRY(dev_malloc_async((void **)&d_off, sizeof(int64_t) * (b->count + 1), s));
+    cudaError_t ce = cudaMemcpyAsync(b->d_mats, mats.data(), sizeof(BatchMat) * b->count, cudaMemcpyHostToDevice, s);
+    if (ce == cudaSuccess)
+        ce = cudaMemcpyAsync(d_off, off.data(), sizeof(int64_t) * (b->count + 1), cudaMemcpyHostToDevice, s);
+    int fst = ce == cudaSuccess ? fill_items((const BatchMat *)b->d_mats, d_off, b->count, b->total_items, b->d_items, s)
+                                : cuda_status(ce, "batch descriptors");
+    cudaFreeAsync(d_off, s);
+    SPMV_TRY(fst);
     SPMV_CUDA_TRY(cudaStreamSynchronize(s));
-    // capture: counter reset + kernel, replayed by spmv_batch_launch
+    // captured once, replayed by spmv_batch_launch
     SPMV_CUDA_TRY(cudaStreamBeginCapture(b->cs, cudaStreamCaptureModeThreadLocal));
-    int st = launch_batch(b, (const BatchMat *)b->d_mats, b->count, b->d_item_off, b->total_items, b->cs);
+    int st = launch_batch(b, (const BatchMat *)b->d_mats, b->d_items, b->total_items, b->cs);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(b->cs, &g);
     if (st != SPMV_OK) {
@@ -386,16 +441,16 @@ int build(spmv_batch *b, cudaStream_t s) {
 }
 
 // median time (us) of `reps` launches of a sub-batch on stream s
-float time_launch(const spmv_batch *b, const BatchMat *mats, int count, const int64_t *off, int64_t total,
-                  cudaStream_t s, int reps, int *status) {
+float time_launch(const spmv_batch *b, const BatchMat *mats, const int2 *items, int64_t total, cudaStream_t s, int reps,
+                  int *status) {
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     std::vector<float> ts;
-    *status = launch_batch(b, mats, count, off, total, s);  // warm-up
+    *status = launch_batch(b, mats, items, total, s);  // warm-up
     for (int r = 0; r < reps && *status == SPMV_OK; ++r) {
         cudaEventRecord(e0, s);
-        *status = launch_batch(b, mats, count, off, total, s);
+        *status = launch_batch(b, mats, items, total, s);
         cudaEventRecord(e1, s);
         cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -473,6 +528,7 @@ int spmv_batch_create(spmv_batch_handle *out, const spmv_handle *hs, int32_t cou
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sm_count, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = dev_malloc((void **)&b->d_counter, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned long long), (cudaStream_t)stream);
     int st = e == cudaSuccess ? SPMV_OK : cuda_status(e, "spmv_batch_create");
     if (st == SPMV_OK) st = build(b, (cudaStream_t)stream);
     if (st != SPMV_OK) {
@@ -558,6 +614,7 @@ int spmv_batch_tune(spmv_batch_handle b, void *stream) {
             M.bsr_val = probe.bsr_val;
             M.bsr_mb = probe.bsr_mb;
             M.bsr_r = probe.bsr_r;
+            M.bsr_s = probe.bsr_s;
             M.n = h->n;
             // the mode is timed on k copies of the matrix in one launch (about
             // 4M entries in all), so that a small matrix is timed at the
@@ -569,6 +626,7 @@ int spmv_batch_tune(spmv_batch_handle b, void *stream) {
             int32_t *meta = nullptr;
             BatchMat *d_m = nullptr;
             int64_t *d_off = nullptr;
+            int2 *d_it = nullptr;
             int st = SPMV_OK;
             if (mode == 0 || mode == BATCH_COO) {
                 st = build_chunk_meta(h, mode, C, &meta, s);
@@ -576,18 +634,21 @@ int spmv_batch_tune(spmv_batch_handle b, void *stream) {
                 if (st == SPMV_OK) st = alloc_partials(&one.part, k * per, 1, one.vt, s);
             }
             M.units = per;
+            M.group = 1;
             std::vector<BatchMat> copies((size_t)k, M);
             std::vector<int64_t> offs((size_t)k + 1);
             for (int64_t r = 0; r <= k; ++r) offs[r] = r * per;
             for (int64_t r = 0; r < k; ++r) copies[r].part_off = mode == 0 || mode == BATCH_COO ? r * per : 0;
             one.count = (int)k;
             if (st == SPMV_OK && (dev_malloc((void **)&d_m, sizeof(BatchMat) * k) != cudaSuccess ||
-                                  dev_malloc((void **)&d_off, sizeof(int64_t) * (k + 1)) != cudaSuccess))
+                                  dev_malloc((void **)&d_off, sizeof(int64_t) * (k + 1)) != cudaSuccess ||
+                                  dev_malloc((void **)&d_it, sizeof(int2) * (size_t)std::max<int64_t>(1, k * per)) != cudaSuccess))
                 st = SPMV_ERR_OOM;
             if (st == SPMV_OK) {
                 cudaMemcpyAsync(d_m, copies.data(), sizeof(BatchMat) * k, cudaMemcpyHostToDevice, s);
                 cudaMemcpyAsync(d_off, offs.data(), sizeof(int64_t) * (k + 1), cudaMemcpyHostToDevice, s);
-                const float t = time_launch(&one, d_m, (int)k, d_off, k * per, s, 3, &st);
+                st = fill_items(d_m, d_off, (int)k, k * per, d_it, s);
+                const float t = st == SPMV_OK ? time_launch(&one, d_m, d_it, k * per, s, 3, &st) : 1e30f;
                 if (st == SPMV_OK && t < best_t) {
                     best_t = t;
                     best_mode = mode;
@@ -597,6 +658,7 @@ int spmv_batch_tune(spmv_batch_handle b, void *stream) {
             dev_free(meta);
             dev_free(d_m);
             dev_free(d_off);
+            dev_free(d_it);
             one.d_counter = nullptr;
             one.cs = nullptr;
             if (st != SPMV_OK) return st;
@@ -614,8 +676,7 @@ int spmv_batch_tune(spmv_batch_handle b, void *stream) {
                 b->group = group;
                 SPMV_TRY(build(b, s));
                 int st = SPMV_OK;
-                const float t = time_launch(b, (const BatchMat *)b->d_mats, b->count, b->d_item_off,
-                                            b->total_items, s, 5, &st);
+                const float t = time_launch(b, (const BatchMat *)b->d_mats, b->d_items, b->total_items, s, 5, &st);
                 SPMV_TRY(st);
                 if (t < best_t) {
                     best_t = t;
