@@ -31,8 +31,8 @@
 // boundaries by cluster barriers.
 //
 // Every dot product is a fixed-shape reduction in fp64, so results are
-// bit-reproducible and every block sees the same alpha and beta.  Vector
-// updates are fused multiply-adds.
+// bit-reproducible and every block sees the same alpha and beta.  fp64 vector
+// updates are fused multiply-adds, fp32 ones round the product and the sum.
 //
 // Termination does not depend on the reductions: the iteration counter grows
 // on every pass and the loop ends once it reaches maxit.
@@ -103,10 +103,13 @@ __device__ double sum_parts(const double *part, int n) {
 __device__ __forceinline__ double wide(double v) { return v; }
 __device__ __forceinline__ double wide(float v) { return (double)v; }
 
-// a + s*b, rounded once: one fp64 instruction where a product and a sum are
-// two (the vector updates of a large fp64 solve are bound by them, not by HBM)
+// a + s*b.  fp64: rounded once, one instruction where a product and a sum are
+// two (the vector updates of a large fp64 solve are bound by them, not by HBM).
+// fp32: the product and the sum rounded separately, so that the fp64 history
+// of r.r stays the one this iteration has always written (fused, it moves in
+// the seventh digit; nothing is gained, fp32 instructions are not scarce).
 __device__ __forceinline__ double axpy1(double a, double s, double b) { return fma(s, b, a); }
-__device__ __forceinline__ float axpy1(float a, float s, float b) { return fmaf(s, b, a); }
+__device__ __forceinline__ float axpy1(float a, float s, float b) { return __fadd_rn(a, __fmul_rn(s, b)); }
 
 template <typename T>
 __global__ void __launch_bounds__(CG_THREADS) k_cg_start(int64_t m, const T *__restrict__ r, const T *__restrict__ b,

@@ -67,3 +67,37 @@ def test_graph_form_in_every_format(oracle, fmt):
 def test_unaligned_iterate(oracle):
     check(oracle, matgen.laplacian_1d(33001), None, shift=1)
     check(oracle, matgen.laplacian_1d(3001), None, shift=1)
+
+
+@pytest.mark.parametrize("m", [1001, 40003])  # the cluster form, the graph form
+def test_fp32_updates_round_product_and_sum(m):
+    """fp32 vector updates round the product and the sum separately: with a
+    diagonal matrix every fp32 step is one numpy rounds the same way, so x is
+    equal bit by bit and the fp64 history differs by the order of its sums
+    only (m terms: under m 2^-53 < 1e-11 of the sum)."""
+    import torch
+    rng = np.random.default_rng(m)
+    d = rng.uniform(1.0, 3.0, m).astype(np.float32)
+    b = rng.standard_normal(m).astype(np.float32)
+    i = np.arange(m, dtype=np.int32)
+    h = create(matgen.Coo(m, m, i, i, d.astype(np.float64)), B.SPMV_F32, B.make_config(format=B.FMT_ELL))
+    steps = 6
+    x = torch.zeros(m, device="cuda")
+    hist = torch.zeros(steps + 1, dtype=torch.float64, device="cuda")
+    try:
+        B.spmv_cg(h, torch.from_numpy(b).cuda(), x, 0.0, steps, hist)
+        torch.cuda.synchronize()
+    finally:
+        B.spmv_destroy(h)
+    dot = lambda u, v: float(np.dot(u.astype(np.float64), v.astype(np.float64)))
+    xs, r, p = np.zeros(m, np.float32), b.copy(), b.copy()
+    rho = [dot(r, r)]
+    for _ in range(steps):
+        q = d * p
+        alpha = np.float32(rho[-1] / dot(p, q))
+        xs = xs + alpha * p
+        r = r + (-alpha) * q
+        rho.append(dot(r, r))
+        p = r + np.float32(rho[-1] / rho[-2]) * p
+    assert np.array_equal(x.cpu().numpy(), xs)
+    assert np.allclose(hist.cpu().numpy(), rho, rtol=1e-11, atol=0.0)
