@@ -38,7 +38,7 @@ struct FeatAcc {
     unsigned long long blocks4;    // nonempty 4x4 blocks
     unsigned long long blocks2;    // nonempty 2x2 blocks
     int min_gap, max_len, max_dist;  // min_gap: 2^31 - 1 minus the shortest row, so that zero starts every field
-    unsigned list_len;               // tiles of heavy block rows listed (one panel's)
+    unsigned list_len;               // entries of the list of heavy block rows (one panel's)
 };
 
 // Row lengths.  A matrix has few distinct lengths, so a histogram of global
@@ -123,10 +123,17 @@ __global__ void __launch_bounds__(ROW_THREADS) k_feat_rows(const int *rowptr, in
 // (380,000 rows, 46M entries) went from 887 to 195 us.
 //
 // A block row of more than `heavy` entries would hold up its warp: it is
-// listed in tiles of HEAVY_TILE entries for k_feat_heavy.
+// listed for k_feat_heavy, once per 32 of its ranges.
 constexpr int FEAT_CAP = 4096;  // most staged entries per warp (one warp per thread block)
+constexpr int FEAT_WARPS = 8;   // warps per SM below which a block row gets more lanes
+constexpr int UNEVEN_LANES = 4;
 constexpr int HEAVY_MIN = 256, HEAVY_MAX = 4096;
-constexpr int HEAVY_THREADS = 256, HEAVY_ITEMS = 8, HEAVY_TILE = HEAVY_THREADS * HEAVY_ITEMS;
+constexpr int HEAVY_THREADS = 128, HEAVY_STRIDE = 32;
+
+// pivots of a row of `len` entries in a heavy block row (k_feat_heavy)
+__device__ __forceinline__ int heavy_pivots(int len) {
+    return (int)(((unsigned)len + HEAVY_STRIDE - 1) / HEAVY_STRIDE);
+}
 
 // sums of one warp into the accumulators
 __device__ __forceinline__ void feat_add(FeatAcc *acc, unsigned long long sd, unsigned dg, unsigned b4, unsigned b2,
@@ -273,7 +280,10 @@ k_feat_groups(const int *__restrict__ rowptr, const int *__restrict__ colidx, in
         __syncwarp();
         const int cnt = b[4] - b[0];
         if (cnt > heavy && sub == 0) {
-            const int nt = (cnt + HEAVY_TILE - 1) / HEAVY_TILE;
+            int pivots = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) pivots += heavy_pivots(b[q + 1] - b[q]);
+            const int nt = (pivots + 31) / 32;
             const unsigned at = atomicAdd(list_len, (unsigned)nt);
             for (int t = 0; t < nt; ++t) list[at + t] = make_int2((int)g, t);
         }
@@ -287,27 +297,27 @@ k_feat_groups(const int *__restrict__ rowptr, const int *__restrict__ colidx, in
     feat_add(acc, sd, dg, b4, b2, md);
 }
 
-// first position in [b, e) whose column is >= c
-__device__ __forceinline__ int lower_col(const int *colidx, int b, int e, int c) {
-    while (b < e) {
-        const int mid = b + ((e - b) >> 1);  // b + e overflows int past 2^30 offsets
-        if (__ldg(colidx + mid) < c) b = mid + 1; else e = mid;
-    }
-    return b;
-}
-
-// The listed tiles of heavy block rows, one thread block each: a thread walks
-// HEAVY_ITEMS consecutive entries and keeps, for each earlier row of the block
-// row, the position its column has reached (columns ascend, so it moves a few
-// entries a step; a much denser earlier row is searched again).  An entry
-// opens a block if neither the entry before it nor an earlier row holds it.
+// The listed heavy block rows, cut into column ranges of a lane each.  Every
+// HEAVY_STRIDE-th entry of each row is a pivot, its column rounded down to a
+// whole 4-column block; a range starts at a pivot and ends at the next larger
+// one of any row, so it holds at most HEAVY_STRIDE + 3 entries of a row however
+// the rows' columns are spread.  The lane of a pivot finds its range by one
+// search per row (the four rows' searches run together) and merges it as
+// k_feat_groups does; where rows share a pivot the first row's lane takes it.
+// With a thread per 8 consecutive entries looking up the earlier rows for each
+// it took 57 us on an R-MAT matrix of scale 17 (a = 0.64), 22 now; whole
+// selection of scale 19 (a = 0.57) 392 and 248.
 __global__ void __launch_bounds__(HEAVY_THREADS)
 k_feat_heavy(const int *__restrict__ rowptr, const int *__restrict__ colidx, int64_t m, int64_t row0,
              const int2 *list, const unsigned *list_len, FeatAcc *acc) {
+    constexpr int S = HEAVY_STRIDE, NONE = 0x7fffffff;
     unsigned long long sd = 0;
     unsigned dg = 0, b4 = 0, b2 = 0;
+    int md = 0;
     const unsigned n = *list_len;
-    for (unsigned it = blockIdx.x; it < n; it += gridDim.x) {
+    const unsigned warp = (blockIdx.x * HEAVY_THREADS + threadIdx.x) >> 5, warps = gridDim.x * (HEAVY_THREADS / 32);
+    auto col = [&](int k) { return __ldg(colidx + k); };
+    for (unsigned it = warp; it < n; it += warps) {
         const int2 item = list[it];
         int b[5];
 #pragma unroll
@@ -315,66 +325,63 @@ k_feat_heavy(const int *__restrict__ rowptr, const int *__restrict__ colidx, int
             const int64_t r = 4 * (int64_t)item.x + q;
             b[q] = __ldg(rowptr + (r < m ? r : m));
         }
-        const int64_t first = (int64_t)b[0] + (int64_t)item.y * HEAVY_TILE + threadIdx.x * HEAVY_ITEMS;
-        if (first >= b[4]) continue;
-        const int k1 = (int)(first + HEAVY_ITEMS < b[4] ? first + HEAVY_ITEMS : b[4]);
-        int row = -1, prev = -1, p[3] = {0, 0, 0};
-#pragma unroll 1
-        for (int k = (int)first; k < k1; ++k) {
-            const int j = __ldg(colidx + k);
-            const int at_row = (k >= b[1]) + (k >= b[2]) + (k >= b[3]);
-            if (at_row != row) {
-                row = at_row;
-                const int start = row == 0 ? b[0] : row == 1 ? b[1] : row == 2 ? b[2] : b[3];
-                prev = k > start ? __ldg(colidx + k - 1) : -1;
+        // this lane's pivot: entry own * S of row `row`
+        int own = item.y * 32 + (threadIdx.x & 31), row = 0;
 #pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if (q < row) p[q] = lower_col(colidx, b[q], b[q + 1], j & ~3);
+        for (int q = 0; q < 3; ++q) {
+            const int pivots = heavy_pivots(b[q + 1] - b[q]);
+            if (row == q && own >= pivots) {
+                own -= pivots;
+                row = q + 1;
             }
-            const int64_t gi = row0 + 4 * (int64_t)item.x + row;
-            const int64_t d = gi > j ? gi - j : j - gi;
-            sd += (unsigned long long)d;
-            dg += d == 0;
-            const bool open2 = prev < 0 || (prev >> 1) != (j >> 1), open4 = prev < 0 || (prev >> 2) != (j >> 2);
-            prev = j;
-            if (!open2) continue;
-            const int c4 = j & ~3, c2 = j & ~1;
-            bool hit4 = false, hit2 = false;
+        }
+        const int rb = row == 0 ? b[0] : row == 1 ? b[1] : row == 2 ? b[2] : b[3];
+        const int re = row == 0 ? b[1] : row == 1 ? b[2] : row == 2 ? b[3] : b[4];
+        if (own >= heavy_pivots(re - rb)) continue;  // past the last row's pivots
+        const int from = col(rb + own * S) & ~3;
+        // first entry of each row at or after column `from`
+        int k[4], e[4];
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                if (q >= row) continue;
-                int at = p[q];
-                const int end = b[q + 1];
-                for (int step = 0; at < end && __ldg(colidx + at) < c4; ++at)
-                    if (++step == 8) {
-                        at = lower_col(colidx, at, end, c4);
-                        break;
-                    }
-                p[q] = at;
-                if (at < end && __ldg(colidx + at) < c4 + 4) {
-                    hit4 = true;
-                    if (q == row - 1 && (row & 1)) {
-                        while (at < end && __ldg(colidx + at) < c2) ++at;  // at most two steps
-                        hit2 = at < end && __ldg(colidx + at) < c2 + 2;
-                    }
+        for (int q = 0; q < 4; ++q) {
+            k[q] = b[q];
+            e[q] = b[q + 1];
+        }
+        while (k[0] < e[0] || k[1] < e[1] || k[2] < e[2] || k[3] < e[3]) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int mid = k[q] + ((e[q] - k[q]) >> 1);
+                if (k[q] < e[q]) {
+                    if (col(mid) < from) k[q] = mid + 1; else e[q] = mid;
                 }
             }
-            b4 += open4 && !hit4;
-            b2 += !hit2;
         }
-    }
-    // the rows' farthest entries
-    int md = 0;
-    for (unsigned it = blockIdx.x; it < n; it += gridDim.x) {
-        const int2 item = list[it];
-        const int64_t r = 4 * (int64_t)item.x + threadIdx.x;
-        if (item.y != 0 || threadIdx.x >= 4 || r >= m) continue;
-        const int s = __ldg(rowptr + r), e = __ldg(rowptr + r + 1);
-        if (s < e) {
-            const int64_t gi = row0 + r, lo = gi - __ldg(colidx + s), hi = __ldg(colidx + e - 1) - gi;
-            md = max(md, (int)max(lo < 0 ? -lo : lo, hi < 0 ? -hi : hi));
+        // the next pivot of any row, and whether an earlier row holds this one
+        int next = NONE;
+        bool mine = true;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            // pivot entry at or after the range's start (offsets in the row: b + S may pass 2^31)
+            const int at = heavy_pivots(k[q] - b[q]), all = heavy_pivots(b[q + 1] - b[q]);
+            int c = at < all ? col(b[q] + at * S) & ~3 : NONE;
+            if (c == from) {
+                mine = mine && q >= row;
+                c = at + 1 < all ? col(b[q] + (at + 1) * S) & ~3 : NONE;
+            }
+            next = min(next, c);
         }
+        if (!mine) continue;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            int lo = k[q], hi = k[q] + min(b[q + 1] - k[q], S + 3);
+            while (lo < hi) {
+                const int mid = lo + ((hi - lo) >> 1);
+                if (col(mid) < next) lo = mid + 1; else hi = mid;
+            }
+            e[q] = lo;
+        }
+        merge_group(col, k, e, row0 + 4 * (int64_t)item.x, sd, dg, b4, b2, md);
     }
+    __syncwarp();
     feat_add(acc, sd, dg, b4, b2, md);
 }
 
@@ -524,13 +531,13 @@ int compute_features(const spmv_matrix *h, double *d_out, cudaStream_t s) {
     const int64_t m = h->m;
     const int maxlen = (int)h->max_row;
     void *buf = nullptr;
-    // histogram, accumulators, list of heavy tiles (one panel's at a time): a
-    // heavy block row has over HEAVY_MIN entries
+    // histogram, accumulators, list of heavy block rows (one panel's at a time): one has
     const int np = h->npanels > 0 ? h->npanels : 1;
     int64_t most = 0;
     for (int p = 0; p < np; ++p) most = std::max(most, h->npanels > 0 ? h->panels[p]->nnz : h->nnz);
     const size_t hist_bytes = (sizeof(unsigned) * ((size_t)maxlen + 1) + 127) / 128 * 128;
-    const size_t list_bytes = sizeof(int2) * (size_t)(most / HEAVY_MIN + most / HEAVY_TILE + 1);
+    // cnt > HEAVY_MIN entries, listed at most cnt / (32 HEAVY_STRIDE) + 2 times
+    const size_t list_bytes = sizeof(int2) * (size_t)(2 * (most / HEAVY_MIN) + most / (32 * HEAVY_STRIDE) + 1);
     SPMV_CUDA_TRY(dev_malloc_async(&buf, hist_bytes + 128 + list_bytes, s));
     unsigned *hist = static_cast<unsigned *>(buf);
     FeatAcc *acc = reinterpret_cast<FeatAcc *>(static_cast<char *>(buf) + hist_bytes);
@@ -558,12 +565,21 @@ int compute_features(const spmv_matrix *h, double *d_out, cudaStream_t s) {
             const int64_t ngroups = (mq + 3) / 4;
             int lpg = 1;
             while (lpg < 32 && 36.0 / lpg * mean4 + 64.0 > FEAT_CAP) lpg *= 2;
+            // ... and, while the chip is not full of warps, more of them with a shorter walk each
+            // (Poisson(22) of 1756 rows: 85 us a selection with one lane, 63 now)
+            while (lpg < 32 && ngroups * lpg < 32 * FEAT_WARPS * sms && mean4 >= 8.0 * lpg) lpg *= 2;
+            // ... or where the longest row of most 32-row groups is far above the mean: a warp is done
+            // when its longest walk is (R-MAT scale 19, whole selection: 248 us with one lane, 204,
+            // 197, 213 with 2, 4, 8)
+            if (csr_uneven(q, 1)) lpg = std::max(lpg, UNEVEN_LANES);
             const int cap = (int)std::min<double>(FEAT_CAP, 128.0 * std::ceil((36.0 / lpg * mean4 + 64.0) / 128.0));
             const int64_t wb = (ngroups + 32 / lpg - 1) / (32 / lpg);
             k_feat_groups<<<(unsigned)(wb < 64 * sms ? wb : 64 * sms), 32, sizeof(int) * (size_t)(cap + 32), s>>>(
                 q->rowptr, q->colidx, mq, row0, heavy, cap, lpg, list, &acc->list_len, acc);
-            k_feat_heavy<<<(unsigned)(4 * sms), HEAVY_THREADS, 0, s>>>(q->rowptr, q->colidx, mq, row0, list,
-                                                                       &acc->list_len, acc);
+            // (a block row holds at most four times the longest row)
+            if (4 * h->max_row > heavy)
+                k_feat_heavy<<<(unsigned)(8 * sms), HEAVY_THREADS, 0, s>>>(q->rowptr, q->colidx, mq, row0, list,
+                                                                           &acc->list_len, acc);
         }
         k_feat_finish<<<1, FIN_THREADS, 0, s>>>(hist, maxlen, m, h->n, h->nnz, acc, d_out);
         if (e == cudaSuccess) e = cudaGetLastError();

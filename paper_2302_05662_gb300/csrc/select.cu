@@ -83,16 +83,25 @@ k_mlp(const double *feat, const float *w, int F, int H, int K, int time_head, in
         }
     }
     __syncthreads();
-    if (t == 0) {
-        int best = 0;
-        float top = lg[0];
-#pragma unroll 8
-        for (int o = 1; o < K; ++o)
+    // the first of the largest logits (a NaN is none), by one warp
+    if (t < 32) {
+        int best = K;
+        float top = -INFINITY;
+        for (int o = t; o < K; o += 32)
             if (lg[o] > top) {
                 top = lg[o];
                 best = o;
             }
-        *choice = best;
+        for (int d = 16; d > 0; d >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, top, d);
+            const int ob = __shfl_xor_sync(0xffffffffu, best, d);
+            if (ov > top || (ov == top && ob < best)) {
+                top = ov;
+                best = ob;
+            }
+        }
+        // a NaN first logit is never passed, and none over -infinity leaves the first
+        if (t == 0) *choice = best == K || lg[0] != lg[0] ? 0 : best;
     }
 }
 
@@ -135,9 +144,11 @@ int run_selector(const spmv_matrix *h, const Selector *sel, cudaStream_t s, doub
     const bool have = sel && sel->K > 0;
     const bool th = have && sel->version >= 2 && logt;
     char *buf = nullptr;
+    // features, choice and times side by side: one copy brings them
     const size_t fb = sizeof(double) * SPMV_NUM_FEATURES;
-    const size_t tb = th ? sizeof(float) * (sel->K + 1) : 0;
-    SPMV_CUDA_TRY(dev_malloc_async((void **)&buf, fb + 16 + tb + 16, s));
+    const size_t tb = th ? sizeof(float) * (sel->K + 1) : 0, all = fb + 16 + tb;
+    SPMV_CUDA_TRY(dev_malloc_async((void **)&buf, all, s));
+    alignas(8) char host[sizeof(double) * SPMV_NUM_FEATURES + 16 + sizeof(float) * (MAX_CLASSES + 1)];
     double *d_f = reinterpret_cast<double *>(buf);
     int *d_c = reinterpret_cast<int *>(buf + fb);
     float *d_t = reinterpret_cast<float *>(buf + fb + 16);
@@ -149,14 +160,17 @@ int run_selector(const spmv_matrix *h, const Selector *sel, cudaStream_t s, doub
             k_mlp<<<1, 256, 0, s>>>(d_f, sel->d_w, sel->F, sel->H, sel->K, th ? 1 : 0, d_c, nullptr,
                                     th ? d_t : nullptr);
             e = cudaGetLastError();
-            if (e == cudaSuccess) e = cudaMemcpyAsync(choice, d_c, sizeof(int), cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess && th) {
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(host, buf, have ? all : fb, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) {
+            std::memcpy(hf, host, fb);
+            if (have) std::memcpy(choice, host + fb, sizeof(int));
+            if (th) {
                 logt->resize(sel->K + 1);
-                e = cudaMemcpyAsync(logt->data(), d_t, tb, cudaMemcpyDeviceToHost, s);
+                std::memcpy(logt->data(), host + fb + 16, tb);
             }
         }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(hf, d_f, fb, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) st = cuda_status(e, "selector");
     }
     cudaFreeAsync(buf, s);

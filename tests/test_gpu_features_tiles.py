@@ -31,6 +31,18 @@ def _rows(lens, n, seed):
     return matgen.Coo(len(lens), n, rows, cols, np.ones(rows.size))
 
 
+def _spans(groups, n):
+    """Block rows of four rows, each (first column, entries, step)."""
+    rows, cols = [], []
+    for i, (first, count, step) in enumerate(r for g in groups for r in g):
+        c = np.arange(first, first + count * step, step)
+        c = c[c < n]
+        rows.append(np.full(c.size, i))
+        cols.append(c)
+    rows, cols = np.concatenate(rows).astype(np.int32), np.concatenate(cols).astype(np.int32)
+    return matgen.Coo(4 * len(groups), n, rows, cols, np.ones(rows.size))
+
+
 CASES = {
     "staged_exactly": lambda: _rows([32] * 128, 600, 1),                 # 32 block rows of 4096 entries in all
     "staged_plus_one": lambda: _rows([32] * 127 + [33], 600, 2),
@@ -49,6 +61,12 @@ CASES = {
     "band": lambda: matgen.banded(3001, 9, np.random.default_rng(10)),
     "power_law": lambda: matgen.rmat(12, 16, np.random.default_rng(11)),
     "long_lengths": lambda: _rows([4095, 4096, 4097, 9000, 1, 0], 10000, 12),  # either side of the shared histogram
+    # enough rows for one lane a block row: 384 staged entries, spans of 384 and 385
+    "one_lane_staged_limit": lambda: _rows([2] * 1280 + [3] * 128 + [2] * 1280 + [3] * 127 + [4] + [2] * 187200, 600, 19),
+    "heavy_strides": lambda: _rows([320, 31, 32, 33, 64, 63, 65, 400, 257, 0, 0, 0, 0, 0, 0, 257, 1, 300], 700, 20),
+    "heavy_clustered": lambda: _spans([[(0, 60000, 7), (30000, 9000, 1), (5, 1, 1), (59999, 1, 1)],
+                                       [(2, 3000, 1), (2, 3000, 1), (1, 3000, 1), (3, 3000, 4)],
+                                       [(1, 400, 3), (0, 1, 1), (600, 500, 2), (20000, 9000, 5)]], 65000),
     "single_entry": lambda: _rows([0, 0, 0, 1], 5, 13),
 }
 
