@@ -66,6 +66,9 @@ __device__ __forceinline__ void ld_group_c(const int *cp, const V *vp, int (&c)[
     if constexpr (GW == 8) {
         ld_idx8_c(cp, c);
         ld_vals8_c(vp, v);
+    } else if constexpr (GW == 1) {  // fp64
+        c[0] = __ldg(cp);
+        v[0] = __ldg(vp);
     } else {
         const int4 w = __ldg(reinterpret_cast<const int4 *>(cp));
         c[0] = w.x; c[1] = w.y; c[2] = w.z; c[3] = w.w;
@@ -106,12 +109,57 @@ __device__ __forceinline__ T csr_lane_range(int a, int b, const int *__restrict_
     return acc;
 }
 
+// Lane `sub` of a row's TPR >= 4 lanes: groups of W entries sub, sub + TPR, ...
+// of the row's entries [s, e), counted from s rounded down to 8 entries, so
+// that no 32-byte sector of the columns is read by two requests (a row read
+// from where it begins reads each sector about twice with four lanes), G
+// groups in flight, the slots outside the row masked.  fp32 and bf16 are
+// bound by loads: four entries a load.  fp64 is bound by its scarce fp64
+// instructions, which masked slots take as well: one entry a load.  us
+// before (W = 1 from the row's beginning, G = 2) / now, default lanes per row:
+//   4 lanes, Poisson(40), 200,000 rows: bf16 55 / 37, fp32 59.5 / 38.9, fp64 64.6 / 51.8
+//   8 lanes, 65-wide band, 2^20 rows: bf16 100 / 98, fp32 128 / 103, fp64 245 / 193
+//   16 lanes, 200 random columns, 200,000 rows: bf16 205 / 169, fp32 196 / 155, fp64 218 / 191
+//   32 lanes, 300 random columns, 100,000 rows: bf16 146 / 137, fp32 151 / 139, fp64 190 / 179
+// With four entries a load fp64 takes 254 us on the band; two a load 238.
+template <typename V, typename T, int TPR, int W, int G>
+__device__ __forceinline__ T csr_lane_groups(int s, int e, int sub, const int *__restrict__ colidx,
+                                             const V *__restrict__ vals, const T *__restrict__ x) {
+    T acc = T(0);
+    for (int k = (s & ~7) + sub * W; k < e; k += TPR * W * G) {
+        int c[G][W];
+        T v[G][W], xv[G][W];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const int q = k + g * TPR * W;
+            const bool any = q < e && q + W > s;
+            if (any) ld_group_c<W>(colidx + q, vals + q, c[g], v[g]);
+#pragma unroll
+            for (int t = 0; t < W; ++t)
+                if (!any || q + t < s || q + t >= e) c[g][t] = -1;
+        }
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int t = 0; t < W; ++t) xv[g][t] = c[g][t] >= 0 ? ld_x(x, c[g][t]) : T(0);
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int t = 0; t < W; ++t)
+                if (c[g][t] >= 0) acc = fma(v[g][t], xv[g][t], acc);
+    }
+    return acc;
+}
+
 // Rows [base, base + 32), or the first `steps` groups of 32 / TPR of them,
 // with TPR lanes per row; the whole warp calls it.
 // With one or two lanes per row each lane sums a contiguous part of its row
 // with 16- or 32-byte loads (csr_lane_range); with more lanes, the lanes of a row
-// take interleaved entries, so a warp's loads of a row are contiguous.
-template <typename V, typename T, int TPR, int UNROLL, int GW = 4>
+// take its groups of entries in turn (csr_lane_groups).
+// W, G: csr_lane_groups'; W = 0: single entries from the row's beginning,
+// UNROLL in flight, for the batched kernel and the register cap of 32 (groups
+// spill there: 96 mixed matrices 264 us with it, 302 with groups)
+template <typename V, typename T, int TPR, int UNROLL, int GW = 4, int W = 0, int G = 1>
 __device__ __forceinline__ void csr_vector_rows(int64_t base, int64_t m, const int *__restrict__ rowptr,
                                                 const int *__restrict__ colidx, const V *__restrict__ vals,
                                                 const T *__restrict__ x, T *__restrict__ y, const Epi<T> &ep,
@@ -139,18 +187,22 @@ __device__ __forceinline__ void csr_vector_rows(int64_t base, int64_t m, const i
                 acc = csr_lane_range<V, T, (UNROLL >= 4 ? 2 : 1), GW>(a, b, colidx, vals, x);
             }
         } else if (!skip) {
-            for (int k = s + sub; k < e; k += TPR * UNROLL) {
-                int c[UNROLL];
-                T v[UNROLL];
+            if constexpr (W > 0) {
+                acc = csr_lane_groups<V, T, TPR, W, G>(s, e, sub, colidx, vals, x);
+            } else {
+                for (int k = s + sub; k < e; k += TPR * UNROLL) {
+                    int c[UNROLL];
+                    T v[UNROLL];
 #pragma unroll
-                for (int u = 0; u < UNROLL; ++u) {
-                    const int kk = k + u * TPR;
-                    c[u] = kk < e ? ld_s(colidx + kk) : -1;
-                    v[u] = kk < e ? ld_val(vals + kk) : T(0);
+                    for (int u = 0; u < UNROLL; ++u) {
+                        const int kk = k + u * TPR;
+                        c[u] = kk < e ? ld_s(colidx + kk) : -1;
+                        v[u] = kk < e ? ld_val(vals + kk) : T(0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < UNROLL; ++u)
+                        if (c[u] >= 0) acc += v[u] * ld_x(x, c[u]);
                 }
-#pragma unroll
-                for (int u = 0; u < UNROLL; ++u)
-                    if (c[u] >= 0) acc += v[u] * ld_x(x, c[u]);
             }
         }
 #pragma unroll
@@ -168,10 +220,14 @@ k_csr_vector(int64_t m, const int *__restrict__ rowptr, const int *__restrict__ 
              const V *__restrict__ vals, const T *__restrict__ x, T *__restrict__ y, T alpha, T beta,
              int long_threshold) {
     const Epi<T> ep(alpha, beta);
+    constexpr bool F64 = sizeof(T) == 8;
+    constexpr int W = REGCAP <= 32 ? 0 : F64 ? 1 : 4;
+    constexpr int U = F64 ? (TPR == 4 ? 4 : 3) : sizeof(V) == 2 && TPR >= 16 ? 3 : 1;
+    constexpr int G = UNROLL < 4 ? U : U == 3 && !F64 ? 4 : 2 * U;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t base = warp * 32; base < m; base += nwarps * 32)
-        csr_vector_rows<V, T, TPR, UNROLL, GW>(base, m, rowptr, colidx, vals, x, y, ep, long_threshold);
+        csr_vector_rows<V, T, TPR, UNROLL, GW, W, G>(base, m, rowptr, colidx, vals, x, y, ep, long_threshold);
 }
 
 // Long CSR rows: one thread block per segment of a long row; segments of one
