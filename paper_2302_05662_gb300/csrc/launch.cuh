@@ -31,10 +31,12 @@ inline int wave_grid(const void *kernel, int threads, int64_t needed_blocks, int
 
 // Scattered columns (under a quarter of consecutive entries in consecutive
 // columns, the layouts' rule) with rows of eight entries and more: all blocks
-// at once for ELL and SELL.  One wave / all blocks, us, SELL: Poisson(16) 2^20
-// rows fp32 69.4 / 65.7, fp64 74.9 / 71.3, R-MAT scale 20 fp32 60.8 / 50.5, fp64
+// at once for ELL, SELL and, from twelve entries on, vector CSR.  One wave /
+// all blocks, us, SELL: Poisson(16) 2^20 rows fp32 69.4 / 65.7, fp64 74.9 / 71.3, R-MAT scale 20 fp32 60.8 / 50.5, fp64
 // 69.5 / 61.7; ELL part of HYB, Poisson(16) fp64 88.3 / 82.1; but Poisson(4) SELL
-// 24.2 / 24.8 and the 27-point stencil fp32 80.3 / 87.9.
+// 24.2 / 24.8 and the 27-point stencil fp32 80.3 / 87.9.  CSR: Poisson(31)
+// 1,600,000 rows fp32 225.4 / 219.0, fp64 252.6 / 242.8, Poisson(60) 400,000 rows
+// fp32 110.5 / 101.4, but Poisson(8.5) 2^20 rows fp64 51.3 / 53.2.
 inline int64_t row_waves(const spmv_matrix *h) {
     return h->contig < 0.25 && h->nnz >= 8 * h->m ? ALL_BLOCKS : ONE_WAVE;
 }
@@ -94,7 +96,8 @@ int launch_csr_vector(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, c
     const int tpb = h->cfg.threads_per_block;
     SPMV_TRY(apply_carveout((const void *)kern, h->cfg.carveout));
     const int64_t rows_per_block = tpb / TPR;
-    const int grid = wave_grid((const void *)kern, tpb, (h->m + rows_per_block - 1) / rows_per_block, h->sm_count);
+    const int grid = wave_grid((const void *)kern, tpb, (h->m + rows_per_block - 1) / rows_per_block, h->sm_count,
+                               h->nnz >= 12 * h->m ? row_waves(h) : ONE_WAVE);
     const int thr = h->lng.nseg > 0 ? (int)h->lng.threshold : 0x7fffffff;
     kern<<<grid, tpb, 0, s>>>(h->m, h->rowptr, h->colidx, (const V *)h->vals, x, y, alpha, beta, thr);
     SPMV_LAUNCH_CHECK();
