@@ -1545,8 +1545,12 @@ int launch_ell_pack(spmv_matrix *h, int64_t width, int64_t pitch, CI *cols, cuda
 // Diagonals instead of columns, where that makes the product read clearly
 // fewer bytes: at most 0.8 of the column-major layout's, and with fp64 values
 // (one multiply-add per slot of a diagonal, entry or not, on the pipe that
-// bounds them) at most 1.06 slots per entry; and from 2^20 entries on: smaller
-// matrices stay in L2, where a product lasts as long as its launch either way.
+// bounds them) at most 1.06 slots per entry; and from 2^20 entries on (a
+// smaller product lasts as long as its launch either way), fp64 from 160 MB of
+// columns and values on: those that stay in L2 (126 MB) do not gain by fewer
+// bytes (27-point stencil, columns / diagonals, us: 216,000 rows 17.3 / 19.6,
+// 300,000 20.8 / 21.8, 400,000 29.9 / 28.3, 1,000,000 61.3 / 56.6; band of 41,
+// 300,000 rows 28.7 / 29.9, 400,000 42.1 / 37.9).
 // A sample of 256 slices says whether it is worth counting them all.  *done:
 // the handle keeps diagonals.
 template <typename V>
@@ -1555,6 +1559,7 @@ int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, boo
     *done = false;
     const int64_t m = h->m, nslices = (m + 32 * R - 1) / (32 * R);
     if (width == 0 || h->nnz < (1 << 20)) return SPMV_OK;
+    if (sizeof(V) == 8 && (double)width * (double)m * (8.0 + index_bytes) < 160e6) return SPMV_OK;
     // staging for a slice's entries: read in place, long rows fall out of L1
     // between steps (band of half-width 32, bf16, 300,000 rows: 198 us a count and
     // 335 a fill with a warp per slice in place, 29 and 147 staged, a warp per 32 rows)

@@ -1,5 +1,5 @@
 """ELL and HYB handles held by diagonals of row slices (2^20 entries and more,
-rows that share their column offsets), against the oracle (gpu_util.TOL) and
+with fp64 values 160 MB of columns and values, rows that share their column offsets), against the oracle (gpu_util.TOL) and
 bit for bit against CSR with one lane per row, which adds a row's entries in
 the same order; matrices just outside the rule keep the column layout."""
 import numpy as np
@@ -32,18 +32,16 @@ def _band(m, n, w, keep=1.0, seed=0):
     return matgen.Coo(m, n, rows, j[ok], rng.standard_normal(rows.size))
 
 
-def _stencil():
-    return matgen.stencil_3d(36, 27, np.random.default_rng(1))          # 46,656 rows, 1.19M entries
-
-
+# f: times the rows (fp64 needs more of them)
 MATS = {
-    "stencil": _stencil,
-    "band": lambda: _band(33333, 33333, 16),
-    "tall": lambda: _band(40001, 30000, 20),                             # the last rows are empty
-    "wide": lambda: _band(34001, 50000, 17),
-    "holes": lambda: _band(33333, 33333, 16, keep=0.98, seed=2),
-    "wide_band": lambda: _band(8200, 8200, 70),                          # 141 diagonals, over 4 rounds of 32
+    "stencil": lambda f: matgen.stencil_3d(36 if f == 1 else 85, 27, np.random.default_rng(1)),  # 46,656 or 614,125 rows
+    "band": lambda f: _band(33333 * f, 33333 * f, 16),
+    "tall": lambda f: _band(40001 * f, 30000 * f, 20),                   # the last rows are empty
+    "wide": lambda f: _band(34001 * f, 50000 * f, 17),
+    "holes": lambda f: _band(33333 * f, 33333 * f, 16, keep=0.98, seed=2),
+    "wide_band": lambda f: _band(8200 * f, 8200 * f, 70),                # 141 diagonals, over 4 rounds of 32
 }
+SCALE = {B.SPMV_F64: 13, B.SPMV_F32: 1, B.SPMV_BF16: 1}
 
 
 def _is_dia(h, vt):
@@ -54,7 +52,7 @@ def _is_dia(h, vt):
 @pytest.mark.parametrize("vt", VTS)
 @pytest.mark.parametrize("name", list(MATS))
 def test_diagonals(oracle, name, vt):
-    coo = MATS[name]()
+    coo = MATS[name](SCALE[vt])
     assert coo.nnz >= 1 << 20
     x = matgen.dense_vector(coo.n, 3)
     y0 = matgen.dense_vector(coo.m, 4)
@@ -77,7 +75,7 @@ def test_diagonals(oracle, name, vt):
 @pytest.mark.parametrize("vt", VTS)
 def test_hyb_part_and_exports(oracle, vt):
     import torch
-    coo = _band(33333, 33333, 16)
+    coo = _band(33333 * SCALE[vt], 33333 * SCALE[vt], 16)
     x = matgen.dense_vector(coo.n, 5)
     for width in (1, 20, 33):
         h = create(coo, vt, B.make_config(format=B.FMT_HYB, hyb_ell_width=width))
@@ -118,7 +116,8 @@ def test_rows_without_an_entry_never_see_its_x():
 @pytest.mark.parametrize("vt", VTS)
 def test_outside_the_rule(oracle, vt):
     """Scattered columns and small matrices keep the column layout."""
-    for coo in (matgen.poisson_rows(70000, 16.0, np.random.default_rng(3)), _band(3000, 3000, 16)):
+    small = _band(33333, 33333, 16) if vt == B.SPMV_F64 else _band(3000, 3000, 16)
+    for coo in (matgen.poisson_rows(70000, 16.0, np.random.default_rng(3)), small):
         x = matgen.dense_vector(coo.n, 8)
         h = create(coo, vt, B.make_config(format=B.FMT_ELL))
         try:
@@ -132,8 +131,8 @@ def test_outside_the_rule(oracle, vt):
 
 def test_batch_of_diagonals(oracle):
     import torch
-    mats = [_stencil(), _band(33333, 33333, 16), _band(500, 500, 3)]
     for vt in VTS:
+        mats = [MATS["stencil"](SCALE[vt]), MATS["band"](SCALE[vt]), _band(500, 500, 3)]
         hs = [create(c, vt, B.make_config(format=B.FMT_ELL)) for c in mats]
         vec = torch.float64 if vt == B.SPMV_F64 else torch.float32
         x = [matgen.dense_vector(c.n, 9) for c in mats]
