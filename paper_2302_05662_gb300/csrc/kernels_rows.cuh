@@ -211,18 +211,21 @@ __device__ __forceinline__ void csr_vector_rows(int64_t base, int64_t m, const i
     }
 }
 
+// groups in flight of a lane of an fp64 row (csr_lane_groups)
+__host__ __device__ constexpr int csr_f64_groups(int tpr) { return tpr == 4 ? 4 : 3; }
+
 // GW: entries per lane load with one or two lanes per row (4: 16-byte
 // loads, 8: 32-byte loads; wider groups read fewer load instructions per
 // entry but mask more slots at a lane's first and last group)
-template <typename V, typename T, int TPR, int UNROLL, int REGCAP, int GW>
+template <typename V, typename T, int TPR, int UNROLL, int REGCAP, int GW, bool GROUPS = true>
 __global__ void __launch_bounds__(1024) __maxnreg__(REGCAP)
 k_csr_vector(int64_t m, const int *__restrict__ rowptr, const int *__restrict__ colidx,
              const V *__restrict__ vals, const T *__restrict__ x, T *__restrict__ y, T alpha, T beta,
              int long_threshold) {
     const Epi<T> ep(alpha, beta);
     constexpr bool F64 = sizeof(T) == 8;
-    constexpr int W = REGCAP <= 32 ? 0 : F64 ? 1 : 4;
-    constexpr int U = F64 ? (TPR == 4 ? 4 : 3) : sizeof(V) == 2 && TPR >= 16 ? 3 : 1;
+    constexpr int W = REGCAP <= 32 || !GROUPS ? 0 : F64 ? 1 : 4;
+    constexpr int U = F64 ? csr_f64_groups(TPR) : sizeof(V) == 2 && TPR >= 16 ? 3 : 1;
     constexpr int G = UNROLL < 4 ? U : U == 3 && !F64 ? 4 : 2 * U;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;

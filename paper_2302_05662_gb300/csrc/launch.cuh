@@ -4,6 +4,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "kernels_rows.cuh"
@@ -90,9 +91,9 @@ int launch_csr_skew(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, cud
     return SPMV_OK;
 }
 
-template <typename V, typename T, int TPR, int U, int RC, int GW>
+template <typename V, typename T, int TPR, int U, int RC, int GW, bool GROUPS = true>
 int launch_csr_vector(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, cudaStream_t s) {
-    auto kern = k_csr_vector<V, T, TPR, U, RC, GW>;
+    auto kern = k_csr_vector<V, T, TPR, U, RC, GW, GROUPS>;
     const int tpb = h->cfg.threads_per_block;
     SPMV_TRY(apply_carveout((const void *)kern, h->cfg.carveout));
     const int64_t rows_per_block = tpb / TPR;
@@ -102,6 +103,20 @@ int launch_csr_vector(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, c
     kern<<<grid, tpb, 0, s>>>(h->m, h->rowptr, h->colidx, (const V *)h->vals, x, y, alpha, beta, thr);
     SPMV_LAUNCH_CHECK();
     return launch_csr_long<V, T>(h, alpha, x, beta, y, s);
+}
+
+// fp64 rows of consecutive columns: the slots a lane steps through, masked ones
+// too, are fp64 instructions and bound it, so groups (csr_lane_groups, begun on
+// average 3.5 entries before the row) are taken where a mean row needs no
+// more of them than single entries from its beginning do.  Bands, us from the
+// beginning / by groups: 33 wide 134.9 / 147.0 (10 and 12 slots), 41 125.5 / 119.8 (12,
+// 12), 45 126.4 / 140.1 (12, 16), 65 163.2 / 136.0 (10, 9), 73 144.6 / 152.1 (10, 12), 81
+// 169.4 / 135.1 (12, 12), 113 144.6 / 129.0 (16, 15).
+inline bool csr_groups(const spmv_matrix *h, int tpr, int unroll) {
+    if (h->vt != SPMV_F64 || h->contig < 0.25 || h->m == 0) return true;
+    const double mean = (double)h->nnz / (double)h->m;
+    const double g = csr_f64_groups(tpr) * (unroll >= 4 ? 2 : 1);
+    return g * std::ceil((mean + 3.5) / (g * tpr)) <= unroll * std::ceil(mean / (unroll * tpr));
 }
 
 // bsr_block selects the load group of one or two lanes per row: 8 entries
@@ -115,6 +130,10 @@ int csr_vector_rc(const spmv_matrix *h, T a, const T *x, T b, T *y, cudaStream_t
         if (h->cfg.bsr_block == 8)
             return h->cfg.regcap == 32 ? launch_csr_vector<V, T, TPR, U, 32, 8>(h, a, x, b, y, s)
                                        : launch_csr_vector<V, T, TPR, U, 64, 8>(h, a, x, b, y, s);
+    }
+    if constexpr (TPR >= 4 && sizeof(T) == 8) {
+        if (h->cfg.regcap != 32 && !csr_groups(h, TPR, U))
+            return launch_csr_vector<V, T, TPR, U, 64, 4, false>(h, a, x, b, y, s);
     }
     return h->cfg.regcap == 32 ? launch_csr_vector<V, T, TPR, U, 32, 4>(h, a, x, b, y, s)
                                : launch_csr_vector<V, T, TPR, U, 64, 4>(h, a, x, b, y, s);

@@ -48,3 +48,19 @@ def test_rows_at_every_offset(oracle, tpr, unroll, regcap, vt):
             assert np.array_equal(got, want)
         else:
             assert rel_err(got, want) <= TOL[vt]
+
+
+@pytest.mark.parametrize("tpr", [4, 8, 16, 32])
+@pytest.mark.parametrize("w", [15, 16, 20, 32, 36, 64])
+def test_fp64_bands_either_side_of_the_rule(oracle, w, tpr):
+    """fp64 rows of consecutive columns: by groups or from their beginning,
+    whichever takes fewer slots at this width (2 w + 1 entries)."""
+    coo = matgen.banded(1501, w, np.random.default_rng(w))
+    x, y0 = matgen.dense_vector(coo.n, 3), matgen.dense_vector(coo.m, 4)
+    for unroll in (1, 2, 4):
+        h = create(coo, B.SPMV_F64, B.make_config(format=B.FMT_CSR, threads_per_row=tpr, unroll=unroll, regcap=64))
+        try:
+            got = run(h, B.SPMV_F64, x, -1.5, 0.5, y0)
+        finally:
+            B.spmv_destroy(h)
+        assert rel_err(got, oracle_for(oracle, coo, B.SPMV_F64, x, -1.5, 0.5, y0)) <= TOL[B.SPMV_F64]
