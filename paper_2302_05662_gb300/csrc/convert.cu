@@ -773,8 +773,10 @@ __global__ void __launch_bounds__(128) k_ell_pack(const int *__restrict__ rowptr
 
 // Diagonals of a slice (32 R rows, of each row its first `width` entries): a
 // merge of the rows' ascending offsets, one step per distinct offset.  Without
-// FILL the steps are counted (given up past `most`), with FILL each step
-// writes its offset, row masks and values.  A block of R warps takes a slice
+// FILL the steps are counted and summed (sums[0], the entries in sums[1]); a
+// slice of more than `most` offsets is given up and counted in sums[2], since
+// its count is then too small to fill by.  With FILL each step writes its
+// offset, row masks and values.  A block of R warps takes a slice
 // (warp w the rows 32 w .. 32 w + 31, a row per lane), every step_s-th slice;
 // the slice's columns and values are staged as in k_ell_pack, at most cap.
 template <typename V, int R, bool FILL>
@@ -789,7 +791,7 @@ k_dia_slices(const int *__restrict__ rowptr, const int *__restrict__ colidx, con
     int *sc = reinterpret_cast<int *>(pack_smem);
     V *sv = reinterpret_cast<V *>(pack_smem + (4 * ell_pack_words(cap) + 15) / 16 * 16);
     if (!FILL && tid == 0) s_entries = 0;
-    unsigned diags = 0, entries = 0;
+    unsigned diags = 0, entries = 0, cut = 0;
     for (int64_t sl = (int64_t)blockIdx.x * step_s; sl < nslices; sl += (int64_t)gridDim.x * step_s) {
         const int64_t first = sl * (32 * R), row = first + tid, end = first + 32 * R < m ? first + 32 * R : m;
         const int w0 = __ldg(rowptr + first), w1 = __ldg(rowptr + end);
@@ -818,7 +820,11 @@ k_dia_slices(const int *__restrict__ rowptr, const int *__restrict__ colidx, con
 #pragma unroll
                 for (int i = 0; i < R; ++i) lo = min(lo, s_min[n & 1][i]);
             }
-            if (lo == INT_MAX || (!FILL && n == most)) break;
+            if (lo == INT_MAX) break;
+            if (!FILL && n == most) {
+                ++cut;
+                break;
+            }
             const bool hit = d == lo;
             if (FILL) {
                 const uint32_t bits = __ballot_sync(FULL, hit);
@@ -847,6 +853,7 @@ k_dia_slices(const int *__restrict__ rowptr, const int *__restrict__ colidx, con
         if (tid == 0) {
             atomicAdd(sums, (unsigned long long)diags);
             atomicAdd(sums + 1, (unsigned long long)s_entries);
+            if (cut) atomicAdd(sums + 2, (unsigned long long)cut);
         }
     }
 }
@@ -1551,8 +1558,9 @@ int launch_ell_pack(spmv_matrix *h, int64_t width, int64_t pitch, CI *cols, cuda
 // bytes (27-point stencil, columns / diagonals, us: 216,000 rows 17.3 / 19.6,
 // 300,000 20.8 / 21.8, 400,000 29.9 / 28.3, 1,000,000 61.3 / 56.6; band of 41,
 // 300,000 rows 28.7 / 29.9, 400,000 42.1 / 37.9).
-// A sample of 256 slices says whether it is worth counting them all.  *done:
-// the handle keeps diagonals.
+// A sample of 256 slices says whether it is worth counting them all.  One slice
+// of more than 4 width + 16 offsets (irregular rows among regular ones) keeps
+// the column layout.  *done: the handle keeps diagonals.
 template <typename V>
 int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, bool *done) {
     constexpr int R = DIA_ROWS<V>;
@@ -1569,14 +1577,14 @@ int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, boo
     };
     Tmp<unsigned long long> sums;
     Tmp<int> count;
-    SPMV_TRY(sums.alloc(2, s));
+    SPMV_TRY(sums.alloc(3, s));
     auto count_kernel = k_dia_slices<V, R, false>;
     SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_of(false)));
     // the diagonals of `slices` slices (one in step_s) and the entries on them
     auto counted = [&](int64_t step_s, int *out, bool *worth) -> int {
         const int64_t slices = (nslices + step_s - 1) / step_s;
-        unsigned long long hs[2];
+        unsigned long long hs[3];
         SPMV_CUDA_TRY(cudaMemsetAsync(sums.p, 0, sizeof(hs), s));
         count_kernel<<<grid1d(slices, 1, 152 * 32), 32 * R, smem_of(false), s>>>(
             h->rowptr, h->colidx, (const V *)h->vals, m, width, nslices, step_s, (int)std::min<int64_t>(4 * width + 16, 1 << 20),
@@ -1586,7 +1594,7 @@ int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, boo
         SPMV_CUDA_TRY(cudaStreamSynchronize(s));
         const double slots = 32.0 * R * (double)hs[0], entries = (double)hs[1];
         const double dia = slots * sizeof(V) + (double)hs[0] * (4 + 4 * R), ell = entries * (double)(sizeof(V) + index_bytes);
-        *worth = entries > 0 && dia <= 0.8 * ell && (sizeof(V) < 8 || slots <= 1.06 * entries);
+        *worth = hs[2] == 0 && entries > 0 && dia <= 0.8 * ell && (sizeof(V) < 8 || slots <= 1.06 * entries);
         return SPMV_OK;
     };
     bool worth = false;
