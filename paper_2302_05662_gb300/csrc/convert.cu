@@ -728,8 +728,23 @@ __device__ __forceinline__ void ell_code(int16_t *p, int c, int64_t r) {
 // 101^3, fp64, 216 us, 156 now (its bytes at the HBM rate: 98), bound by
 // load latency at the 20 warps per SM that the staging leaves room for.
 // One padding word per 32 spreads rows of one length over the banks.
-constexpr int ELL_PACK_CAP = 4608, ELL_PACK_SMEM = 96 * 1024, DIA_PACK_CAP = 20480;
-__host__ __device__ inline size_t ell_pack_words(int cap) { return (size_t)cap + cap / 32 + 1; }
+constexpr int ELL_PACK_CAP = 4608, ELL_PACK_SMEM = 96 * 1024;
+__host__ __device__ constexpr size_t ell_pack_words(int cap) { return (size_t)cap + cap / 32 + 1; }
+
+// Entries of a slice that k_dia_slices stages, at most: 20480, less where their
+// columns and values (12 bytes an entry for fp64) would not fit in the 227 KB a
+// block may have.  A slice of more entries is read in place.
+constexpr size_t DIA_PACK_SMEM = 224 * 1024;
+template <typename V>
+constexpr size_t dia_pack_smem(int cap, bool values) {
+    return (4 * ell_pack_words(cap) + 15) / 16 * 16 + (values ? sizeof(V) * ell_pack_words(cap) : 0);
+}
+template <typename V>
+constexpr int dia_pack_cap() {
+    int cap = 20480;
+    while (dia_pack_smem<V>(cap, true) > DIA_PACK_SMEM) cap -= 32;
+    return cap;
+}
 
 template <typename V, typename CI>
 __global__ void __launch_bounds__(128) k_ell_pack(const int *__restrict__ rowptr, const int *__restrict__ colidx,
@@ -1571,10 +1586,8 @@ int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, boo
     // staging for a slice's entries: read in place, long rows fall out of L1
     // between steps (band of half-width 32, bf16, 300,000 rows: 198 us a count and
     // 335 a fill with a warp per slice in place, 29 and 147 staged, a warp per 32 rows)
-    const int cap = (int)std::min<int64_t>(DIA_PACK_CAP, 32 * R * width);
-    auto smem_of = [&](bool values) {
-        return (4 * ell_pack_words(cap) + 15) / 16 * 16 + (values ? sizeof(V) * ell_pack_words(cap) : 0);
-    };
+    const int cap = (int)std::min<int64_t>(dia_pack_cap<V>(), 32 * R * width);
+    auto smem_of = [&](bool values) { return dia_pack_smem<V>(cap, values); };
     Tmp<unsigned long long> sums;
     Tmp<int> count;
     SPMV_TRY(sums.alloc(3, s));
