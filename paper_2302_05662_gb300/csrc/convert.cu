@@ -1543,6 +1543,14 @@ void free_packed(spmv_matrix *h) {
 
 namespace {
 
+// The most dynamic shared memory a kernel is ever launched with.  Always the
+// same amount for a kernel: the limit is the process's, and a thread that set
+// it to what its own launch needs would take from another thread's.
+int allow_smem(const void *kernel, size_t most) {
+    SPMV_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+    return SPMV_OK;
+}
+
 template <typename V, typename CI>
 int launch_ell_pack_t(spmv_matrix *h, int64_t width, int64_t pitch, CI *cols, cudaStream_t s) {
     auto kern = k_ell_pack<V, CI>;
@@ -1550,7 +1558,7 @@ int launch_ell_pack_t(spmv_matrix *h, int64_t width, int64_t pitch, CI *cols, cu
     const size_t per_warp = ell_pack_words(cap) * (sizeof(V) + 4);
     const int nw = (int)std::max<size_t>(1, std::min<size_t>(4, ELL_PACK_SMEM / per_warp));
     const size_t smem = (sizeof(V) * ell_pack_words(cap) * nw + 15) / 16 * 16 + 4 * ell_pack_words(cap) * nw;
-    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SPMV_TRY(allow_smem((const void *)kern, ELL_PACK_SMEM));
     kern<<<grid1d(pitch, 32 * nw, 1 << 20), 32 * nw, smem, s>>>(h->rowptr, h->colidx, (const V *)h->vals, h->m, width,
                                                                 pitch, cap, cols, (V *)h->ell_val);
     SPMV_CUDA_TRY(cudaGetLastError());
@@ -1592,8 +1600,7 @@ int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, boo
     Tmp<int> count;
     SPMV_TRY(sums.alloc(3, s));
     auto count_kernel = k_dia_slices<V, R, false>;
-    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem_of(false)));
+    SPMV_TRY(allow_smem((const void *)count_kernel, DIA_PACK_SMEM));
     // the diagonals of `slices` slices (one in step_s) and the entries on them
     auto counted = [&](int64_t step_s, int *out, bool *worth) -> int {
         const int64_t slices = (nslices + step_s - 1) / step_s;
@@ -1626,8 +1633,7 @@ int pack_dia(spmv_matrix *h, int64_t width, int index_bytes, cudaStream_t s, boo
     SPMV_TRY(dalloc_slab({slab_bytes(&h->dia_val, sizeof(V) * (size_t)total * 32 * R), slab(&h->dia_off, (size_t)total),
                           slab(&h->dia_mask, (size_t)total * R)}));
     auto fill = k_dia_slices<V, R, true>;
-    SPMV_CUDA_TRY(cudaFuncSetAttribute((const void *)fill, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem_of(true)));
+    SPMV_TRY(allow_smem((const void *)fill, DIA_PACK_SMEM));
     fill<<<grid1d(nslices, 1, 1 << 30), 32 * R, smem_of(true), s>>>(h->rowptr, h->colidx, (const V *)h->vals, m, width, nslices, 1,
                                                              INT_MAX, cap, h->dia_ptr, nullptr, nullptr, h->dia_off,
                                                              h->dia_mask, (V *)h->dia_val);
