@@ -19,13 +19,14 @@ int resident_blocks(const void *kernel, int threads);
 // One wave is best where every warp's share takes the same time: blocks start
 // once and their loads follow each other without a gap.  Where shares differ
 // (gathers that miss at random, uneven rows) a fixed share leaves the chip
-// waiting for its slowest warps, and blocks handed out as others end balance it
-// (from three waves of them on: Poisson(40) 200,000 rows SELL fp32, 1.3 waves, 30.6
-// us in one wave, 35.6 with all blocks).
+// waiting for its slowest warps, and blocks handed out as others end balance it,
+// from `from` waves of them on (SELL: Poisson(40) 200,000 rows fp32, 1.3 waves,
+// 30.6 us in one wave, 35.6 with all blocks).
 constexpr int64_t ONE_WAVE = 1, ALL_BLOCKS = int64_t(1) << 30;
-inline int wave_grid(const void *kernel, int threads, int64_t needed_blocks, int sm_count, int64_t waves = ONE_WAVE) {
+inline int wave_grid(const void *kernel, int threads, int64_t needed_blocks, int sm_count, int64_t waves = ONE_WAVE,
+                     double from = 3.0) {
     int64_t cap = (int64_t)resident_blocks(kernel, threads) * sm_count;
-    if (needed_blocks >= 3 * cap) cap = std::min<int64_t>(cap * waves, 0x7fffffff);
+    if ((double)needed_blocks >= from * (double)cap) cap = std::min<int64_t>(cap * waves, 0x7fffffff);
     int64_t g = needed_blocks < cap ? needed_blocks : cap;
     return (int)(g < 1 ? 1 : g);
 }
@@ -35,9 +36,12 @@ inline int wave_grid(const void *kernel, int threads, int64_t needed_blocks, int
 // at once for ELL, SELL and, from twelve entries on, vector CSR.  One wave /
 // all blocks, us, SELL: Poisson(16) 2^20 rows fp32 69.4 / 65.7, fp64 74.9 / 71.3, R-MAT scale 20 fp32 60.8 / 50.5, fp64
 // 69.5 / 61.7; ELL part of HYB, Poisson(16) fp64 88.3 / 82.1; but Poisson(4) SELL
-// 24.2 / 24.8 and the 27-point stencil fp32 80.3 / 87.9.  CSR: Poisson(31)
-// 1,600,000 rows fp32 225.4 / 219.0, fp64 252.6 / 242.8, Poisson(60) 400,000 rows
-// fp32 110.5 / 101.4, but Poisson(8.5) 2^20 rows fp64 51.3 / 53.2.
+// 24.2 / 24.8 and the 27-point stencil fp32 80.3 / 87.9.  CSR, from 1.5 waves on:
+// 1.07 waves (250,000 rows) Poisson(40) fp32 45.3 / 50.0, Poisson(100) fp64 135.2 /
+// 141.0; 1.7 waves (400,000) fp32 Poisson(24) 49.3 / 45.2, (40) 77.7 / 71.7, (60) 110.7 /
+// 101.1, fp64 (100) 204.9 / 182.4; 2.1 waves fp64 (24) 55.4 / 57.4, (40) 86.2 / 86.3, (60)
+// 127.4 / 123.9; 4.3 waves (1,000,000) fp32 (24) 110.9 / 104.6, fp64 (14) 82.9 / 78.6; but
+// Poisson(8.5) 2^20 rows fp64 51.3 / 53.2.
 inline int64_t row_waves(const spmv_matrix *h) {
     return h->contig < 0.25 && h->nnz >= 8 * h->m ? ALL_BLOCKS : ONE_WAVE;
 }
@@ -96,9 +100,9 @@ int launch_csr_vector(const spmv_matrix *h, T alpha, const T *x, T beta, T *y, c
     auto kern = k_csr_vector<V, T, TPR, U, RC, GW, GROUPS>;
     const int tpb = h->cfg.threads_per_block;
     SPMV_TRY(apply_carveout((const void *)kern, h->cfg.carveout));
-    const int64_t rows_per_block = tpb / TPR;
-    const int grid = wave_grid((const void *)kern, tpb, (h->m + rows_per_block - 1) / rows_per_block, h->sm_count,
-                               h->nnz >= 12 * h->m ? row_waves(h) : ONE_WAVE);
+    // a warp takes 32 rows whatever the lanes per row, so a block takes tpb of them
+    const int grid = wave_grid((const void *)kern, tpb, (h->m + tpb - 1) / tpb, h->sm_count,
+                               h->nnz >= 12 * h->m ? row_waves(h) : ONE_WAVE, 1.5);
     const int thr = h->lng.nseg > 0 ? (int)h->lng.threshold : 0x7fffffff;
     kern<<<grid, tpb, 0, s>>>(h->m, h->rowptr, h->colidx, (const V *)h->vals, x, y, alpha, beta, thr);
     SPMV_LAUNCH_CHECK();
