@@ -3,11 +3,9 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
-#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <mutex>
-#include <unordered_map>
 #include <utility>
 #include <vector>
 
@@ -18,210 +16,11 @@ namespace spmv {
 
 namespace {
 thread_local char g_err[512] = "";
-thread_local long long g_alloc_count = 0;
-
-// SPMV_FAULT_ALLOC=k (k >= 1): the k-th allocation of each entry-point call
-// fails; read on every allocation so a test can set and clear it at will
-bool fault_injected() {
-    const char *v = std::getenv("SPMV_FAULT_ALLOC");
-    ++g_alloc_count;
-    if (!v || !*v) return false;
-    const long long k = std::atoll(v);
-    return k > 0 && g_alloc_count == k;
-}
 }  // namespace
 
 void entry_reset() {
     g_err[0] = 0;
-    g_alloc_count = 0;
-}
-
-// ---------------------------------------------------------------------------
-// Device memory.  A cudaMalloc and cudaFree pair costs 70 us and more, and a
-// handle holds up to twenty small arrays (work items, join scratch, row
-// pointers of small matrices), so blocks of up to SMALL_MOST bytes are kept:
-// a freed block waits until a real cudaFree of the library has come back
-// (which waits for all work on the device, as freeing it would have) and is
-// then handed out again.  Temporaries of one call come from a stream-ordered
-// pool of the library that keeps POOL_KEEP bytes mapped across the call's own
-// synchronisations (the default pool unmaps at each: 2 us per MB to map and
-// unmap).  At most SMALL_KEEP + POOL_KEEP bytes are kept per device (0.1% of
-// it); what exceeds them goes back at once, the rest when an allocation fails.
-// ---------------------------------------------------------------------------
-namespace {
-constexpr size_t SMALL_MOST = size_t(8) << 20, SMALL_KEEP = size_t(64) << 20, POOL_KEEP = size_t(256) << 20;
-
-struct Block {
-    size_t size;  // 0: larger than SMALL_MOST, not kept
-    int dev;
-};
-std::mutex g_mem_mu;
-std::unordered_map<void *, Block> g_blocks;                         // every block handed out or kept
-std::map<std::pair<int, size_t>, std::vector<void *>> g_ready;      // kept blocks by (device, size)
-std::map<int, std::vector<void *>> g_waiting;                       // freed since the device's last real cudaFree
-std::map<int, size_t> g_kept;                                       // bytes in the two
-std::map<int, cudaMemPool_t> g_pools;
-
-// four sizes an octave: at most a quarter more than asked for
-size_t block_size(size_t bytes) {
-    size_t s = 256;
-    while (s < bytes) s *= 2;
-    if (s <= 256) return s;
-    const size_t quarter = s / 8;
-    size_t t = s / 2;
-    while (t < bytes) t += quarter;
-    return (t + 255) / 256 * 256;
-}
-
-// (lock held) a real cudaFree of device dev has come back: what was freed before it is idle
-void waited(int dev) try {
-    auto &w = g_waiting[dev];
-    for (; !w.empty(); w.pop_back()) g_ready[{dev, g_blocks[w.back()].size}].push_back(w.back());
-} catch (const std::bad_alloc &) {  // the rest goes on waiting
-}
-
-// (lock held) frees a block for good
-void free_now(void *p, int dev) {
-    g_blocks.erase(p);
-    cudaFree(p);
-    waited(dev);
-}
-
-// (lock held) gives back everything kept on a device
-void give_back(int dev) {
-    auto w = g_waiting.find(dev);
-    if (w != g_waiting.end() && !w->second.empty()) {
-        void *q = w->second.back();
-        w->second.pop_back();
-        free_now(q, dev);
-    }
-    for (auto &r : g_ready) {
-        if (r.first.first != dev) continue;
-        for (void *q : r.second) {
-            g_blocks.erase(q);
-            cudaFree(q);
-        }
-        r.second.clear();
-    }
-    g_kept[dev] = 0;
-    auto pool = g_pools.find(dev);
-    if (pool != g_pools.end() && pool->second) cudaMemPoolTrimTo(pool->second, 0);
-}
-
-// (lock held) the library's pool of a device; null where it cannot be made
-cudaMemPool_t pool_of(int dev) {
-    auto it = g_pools.find(dev);
-    if (it != g_pools.end()) return it->second;
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    cudaMemPool_t pool = nullptr;
-    uint64_t keep = POOL_KEEP;
-    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
-        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-        cudaGetLastError();
-        pool = nullptr;
-    }
-    g_pools[dev] = pool;
-    return pool;
-}
-}  // namespace
-
-cudaError_t dev_malloc(void **p, size_t bytes) try {
-    *p = nullptr;
-    if (fault_injected()) return cudaErrorMemoryAllocation;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const size_t size = bytes <= SMALL_MOST ? block_size(bytes) : 0;
-    std::lock_guard<std::mutex> lk(g_mem_mu);
-    if (size) {
-        auto &ready = g_ready[{dev, size}];
-        auto &waiting = g_waiting[dev];
-        if (ready.empty()) {
-            // blocks of the size are waiting: one real cudaFree (of the smallest waiting) makes them ready
-            size_t same = 0, least = 0;
-            for (size_t i = 0; i < waiting.size(); ++i) {
-                same += g_blocks[waiting[i]].size == size;
-                if (g_blocks[waiting[i]].size < g_blocks[waiting[least]].size) least = i;
-            }
-            if (same > (same && g_blocks[waiting[least]].size == size ? 1u : 0u)) {
-                void *q = waiting[least];
-                waiting.erase(waiting.begin() + least);
-                g_kept[dev] -= g_blocks[q].size;
-                free_now(q, dev);
-            }
-        }
-        if (!ready.empty()) {
-            *p = ready.back();
-            ready.pop_back();
-            g_kept[dev] -= size;
-            return cudaSuccess;
-        }
-    }
-    e = cudaMalloc(p, size ? size : bytes);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        give_back(dev);
-        e = cudaMalloc(p, size ? size : bytes);
-    }
-    if (e != cudaSuccess) *p = nullptr;
-    else g_blocks[*p] = Block{size, dev};
-    return e;
-} catch (const std::bad_alloc &) {  // of the host's tables
-    if (*p) cudaFree(*p);
-    *p = nullptr;
-    return cudaErrorMemoryAllocation;
-}
-
-void dev_free(void *p) {
-    if (!p) return;
-    std::lock_guard<std::mutex> lk(g_mem_mu);
-    auto it = g_blocks.find(p);
-    const Block b = it == g_blocks.end() ? Block{0, 0} : it->second;
-    try {
-        if (b.size && g_kept[b.dev] + b.size <= SMALL_KEEP) {
-            g_waiting[b.dev].push_back(p);
-            g_kept[b.dev] += b.size;
-            return;
-        }
-    } catch (const std::bad_alloc &) {
-    }
-    free_now(p, b.dev);
-}
-
-cudaError_t dev_malloc_async(void **p, size_t bytes, cudaStream_t s) try {
-    *p = nullptr;
-    if (fault_injected()) return cudaErrorMemoryAllocation;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    cudaMemPool_t pool;
-    {
-        std::lock_guard<std::mutex> lk(g_mem_mu);
-        pool = pool_of(dev);
-    }
-    if (!pool) return cudaMallocAsync(p, bytes, s);
-    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        {
-            std::lock_guard<std::mutex> lk(g_mem_mu);
-            give_back(dev);
-        }
-        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-    }
-    return e;
-} catch (const std::bad_alloc &) {
-    return cudaErrorMemoryAllocation;
-}
-
-void dev_free_waiting(void *p) {
-    if (!p) return;
-    std::lock_guard<std::mutex> lk(g_mem_mu);
-    auto it = g_blocks.find(p);
-    free_now(p, it == g_blocks.end() ? 0 : it->second.dev);
+    reset_alloc_count();
 }
 
 void set_error(const char *fmt, ...) {
@@ -461,8 +260,8 @@ void destroy_all(spmv_matrix *h) {
     free_packed(h);
     dev_free(h->rowptr);
     dev_free(h->vals);  // and the columns behind them
-    // a real cudaFree: waits for work still using the arrays, which may then be handed out again
-    dev_free_waiting(h->d_status);
+    dev_free(h->d_status);
+    dev_settle();  // waits for work still using the arrays, which may then be handed out again
     h->d_status = nullptr;
     h->rowptr = h->colidx = nullptr;
     h->vals = nullptr;
@@ -632,7 +431,7 @@ int spmv_create(spmv_handle *out, int64_t m, int64_t n, int64_t nnz, const int32
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_status, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) {
         int st = cuda_status(e, "device query");
-        dev_free_waiting(h->d_status);
+        dev_free(h->d_status);
         delete h;
         return st;
     }

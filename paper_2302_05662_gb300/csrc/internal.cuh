@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <vector>
 
+#include "memory.cuh"
 #include "spmv.h"
 
 namespace spmv {
@@ -20,30 +21,9 @@ namespace spmv {
 void set_error(const char *fmt, ...);
 int cuda_status(cudaError_t e, const char *what);
 
-// Every device allocation of the library goes through these two, so that
-// the host-side fault injector can fail one of them: with the environment
-// variable SPMV_FAULT_ALLOC=k, the k-th allocation of an entry-point call
-// returns cudaErrorMemoryAllocation without allocating (the call must then
-// return SPMV_ERR_OOM and release what it had allocated).  entry_reset(),
-// called first by every entry point that allocates, clears the thread's
-// error message and its allocation count.
-cudaError_t dev_malloc(void **p, size_t bytes);
-cudaError_t dev_malloc_async(void **p, size_t bytes, cudaStream_t s);
-template <typename T>
-inline cudaError_t dev_malloc(T **p, size_t bytes) {
-    return dev_malloc(reinterpret_cast<void **>(p), bytes);
-}
-template <typename T>
-inline cudaError_t dev_malloc_async(T **p, size_t bytes, cudaStream_t s) {
-    return dev_malloc_async(reinterpret_cast<void **>(p), bytes, s);
-}
+// called first by every entry point that allocates: clears the thread's error
+// message and its allocation count (memory.cuh)
 void entry_reset();
-
-// Frees what dev_malloc gave (null is fine).  The block may still be in use by
-// work already launched: it is handed out again only after a real cudaFree.
-// dev_free_waiting is that: it returns once the device's work is done.
-void dev_free(void *p);
-void dev_free_waiting(void *p);
 
 #define SPMV_CUDA_TRY(expr)                                       \
     do {                                                          \

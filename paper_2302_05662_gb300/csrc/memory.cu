@@ -1,0 +1,234 @@
+// Device memory (memory.cuh).
+//
+// A cudaMalloc and cudaFree pair costs 70 us and more, and a handle holds up
+// to twenty small arrays (work items, join scratch, row pointers of small
+// matrices), so blocks of up to SMALL_MOST bytes are kept: a freed block waits
+// until the library has waited for the device (work launched before the free
+// may still use it) and is then handed out again.  Where that wait fails, the
+// blocks go on waiting.  Temporaries of one call come from a stream-ordered
+// pool of the library that keeps POOL_KEEP bytes mapped across the call's own
+// synchronisations (the default pool unmaps at each: 2 us per MB to map and
+// unmap).  At most SMALL_KEEP + POOL_KEEP bytes are kept per device (0.1% of
+// it); what exceeds them goes back at once, the rest when an allocation fails.
+#include "memory.cuh"
+
+#include <cstdint>
+#include <cstdlib>
+#include <map>
+#include <mutex>
+#include <new>
+#include <unordered_map>
+#include <utility>
+#include <vector>
+
+namespace spmv {
+
+namespace {
+
+thread_local long long g_alloc_count = 0;
+
+// read on every allocation so a test can set and clear it at will
+bool fault_injected() {
+    const char *v = std::getenv("SPMV_FAULT_ALLOC");
+    ++g_alloc_count;
+    if (!v || !*v) return false;
+    const long long k = std::atoll(v);
+    return k > 0 && g_alloc_count == k;
+}
+
+constexpr size_t SMALL_MOST = size_t(8) << 20, SMALL_KEEP = size_t(64) << 20, POOL_KEEP = size_t(256) << 20;
+
+struct Block {
+    size_t size;
+    int dev;
+};
+// what is kept of one device
+struct Kept {
+    std::map<size_t, std::vector<void *>> ready;      // idle blocks by size
+    std::vector<std::pair<size_t, void *>> waiting;   // freed since the device was last waited for
+    size_t bytes = 0;                                 // in the two
+    cudaMemPool_t pool = nullptr;
+    bool pool_tried = false;
+};
+std::mutex g_mem_mu;
+std::unordered_map<void *, Block> g_blocks;  // every small block handed out or kept
+std::map<int, Kept> g_kept;                  // by device
+
+// four sizes an octave: at most a quarter more than asked for
+size_t block_size(size_t bytes) {
+    size_t s = 256;
+    while (s < bytes) s *= 2;
+    if (s <= 256) return s;
+    const size_t quarter = s / 8;
+    size_t t = s / 2;
+    while (t < bytes) t += quarter;
+    return (t + 255) / 256 * 256;
+}
+
+// a failure leaves no error behind for the next launch's check
+void free_now(void *p) {
+    if (cudaFree(p) != cudaSuccess) cudaGetLastError();
+}
+
+// (lock held) waits for the device, then makes the blocks freed before ready
+void settle(int dev) {
+    auto it = g_kept.find(dev);
+    if (it == g_kept.end() || it->second.waiting.empty()) return;
+    if (cudaDeviceSynchronize() != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    Kept &k = it->second;
+    try {
+        for (; !k.waiting.empty(); k.waiting.pop_back()) k.ready[k.waiting.back().first].push_back(k.waiting.back().second);
+    } catch (const std::bad_alloc &) {  // the rest goes on waiting
+    }
+}
+
+// (lock held) a ready block of the size, or null; *waits: blocks of the size are waiting
+void *take(int dev, size_t size, bool *waits) {
+    *waits = false;
+    auto it = g_kept.find(dev);
+    if (it == g_kept.end()) return nullptr;
+    Kept &k = it->second;
+    auto r = k.ready.find(size);
+    if (r != k.ready.end() && !r->second.empty()) {
+        void *p = r->second.back();
+        r->second.pop_back();
+        k.bytes -= size;
+        return p;
+    }
+    for (const auto &w : k.waiting) *waits = *waits || w.first == size;
+    return nullptr;
+}
+
+// (lock held) gives back everything kept on a device
+void give_back(int dev) {
+    auto it = g_kept.find(dev);
+    if (it == g_kept.end()) return;
+    Kept &k = it->second;
+    for (auto &r : k.ready)
+        for (void *p : r.second) {
+            g_blocks.erase(p);
+            free_now(p);
+        }
+    for (const auto &w : k.waiting) {
+        g_blocks.erase(w.second);
+        free_now(w.second);
+    }
+    k.ready.clear();
+    k.waiting.clear();
+    k.bytes = 0;
+    if (k.pool) cudaMemPoolTrimTo(k.pool, 0);
+}
+
+// (lock held) the library's pool of a device; null where it cannot be made
+cudaMemPool_t pool_of(int dev) {
+    Kept &k = g_kept[dev];
+    if (k.pool_tried) return k.pool;
+    k.pool_tried = true;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    uint64_t keep = POOL_KEEP;
+    if (cudaMemPoolCreate(&k.pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(k.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        k.pool = nullptr;
+    }
+    return k.pool;
+}
+
+}  // namespace
+
+void reset_alloc_count() { g_alloc_count = 0; }
+
+cudaError_t dev_malloc(void **p, size_t bytes) {
+    *p = nullptr;
+    if (fault_injected()) return cudaErrorMemoryAllocation;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const size_t size = bytes <= SMALL_MOST ? block_size(bytes) : 0;
+    std::lock_guard<std::mutex> lk(g_mem_mu);
+    if (size) {
+        bool waits = false;
+        *p = take(dev, size, &waits);
+        if (!*p && waits) {
+            settle(dev);
+            *p = take(dev, size, &waits);
+        }
+        if (*p) return cudaSuccess;
+    }
+    e = cudaMalloc(p, size ? size : bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        give_back(dev);
+        e = cudaMalloc(p, size ? size : bytes);
+    }
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        return e;
+    }
+    if (size) try {
+            g_blocks[*p] = Block{size, dev};
+        } catch (const std::bad_alloc &) {  // unlisted: goes back at once when freed
+        }
+    return e;
+}
+
+void dev_free(void *p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> lk(g_mem_mu);
+    auto it = g_blocks.find(p);
+    if (it != g_blocks.end()) {
+        const Block b = it->second;
+        try {
+            Kept &k = g_kept[b.dev];
+            if (k.bytes + b.size <= SMALL_KEEP) {
+                k.waiting.emplace_back(b.size, p);
+                k.bytes += b.size;
+                return;
+            }
+        } catch (const std::bad_alloc &) {
+        }
+        g_blocks.erase(it);
+    }
+    free_now(p);
+}
+
+void dev_settle() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    std::lock_guard<std::mutex> lk(g_mem_mu);
+    settle(dev);
+}
+
+cudaError_t dev_malloc_async(void **p, size_t bytes, cudaStream_t s) try {
+    *p = nullptr;
+    if (fault_injected()) return cudaErrorMemoryAllocation;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lk(g_mem_mu);
+        pool = pool_of(dev);
+    }
+    if (!pool) return cudaMallocAsync(p, bytes, s);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        {
+            std::lock_guard<std::mutex> lk(g_mem_mu);
+            give_back(dev);
+        }
+        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    }
+    return e;
+} catch (const std::bad_alloc &) {
+    return cudaErrorMemoryAllocation;
+}
+
+}  // namespace spmv
