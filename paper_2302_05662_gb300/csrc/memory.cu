@@ -50,7 +50,7 @@ struct Kept {
     cudaMemPool_t pool = nullptr;
     bool pool_tried = false;
 };
-std::mutex g_mem_mu;
+std::mutex g_mem_mu;  // guards the tables; not held while the device is waited for or memory mapped
 std::unordered_map<void *, Block> g_blocks;  // every small block handed out or kept
 std::map<int, Kept> g_kept;                  // by device
 
@@ -70,24 +70,37 @@ void free_now(void *p) {
     if (cudaFree(p) != cudaSuccess) cudaGetLastError();
 }
 
-// (lock held) waits for the device, then makes the blocks freed before ready
+// waits for the device, then makes the blocks freed before the wait ready
 void settle(int dev) {
-    auto it = g_kept.find(dev);
-    if (it == g_kept.end() || it->second.waiting.empty()) return;
-    if (cudaDeviceSynchronize() != cudaSuccess) {
-        cudaGetLastError();
-        return;
+    std::vector<std::pair<size_t, void *>> w;
+    {
+        std::lock_guard<std::mutex> lk(g_mem_mu);
+        auto it = g_kept.find(dev);
+        if (it == g_kept.end() || it->second.waiting.empty()) return;
+        w.swap(it->second.waiting);
     }
-    Kept &k = it->second;
-    try {
-        for (; !k.waiting.empty(); k.waiting.pop_back()) k.ready[k.waiting.back().first].push_back(k.waiting.back().second);
-    } catch (const std::bad_alloc &) {  // the rest goes on waiting
+    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+    if (!idle) cudaGetLastError();
+    size_t left = 0;  // blocks the host has no memory to list: they go back
+    {
+        std::lock_guard<std::mutex> lk(g_mem_mu);
+        Kept &k = g_kept.find(dev)->second;
+        for (const auto &b : w) try {
+                if (idle) k.ready[b.first].push_back(b.second);
+                else k.waiting.push_back(b);
+            } catch (const std::bad_alloc &) {
+                k.bytes -= b.first;
+                g_blocks.erase(b.second);
+                w[left++] = b;
+            }
     }
+    for (size_t i = 0; i < left; ++i) free_now(w[i].second);
 }
 
-// (lock held) a ready block of the size, or null; *waits: blocks of the size are waiting
+// a ready block of the size, or null; *waits: blocks of the size are waiting
 void *take(int dev, size_t size, bool *waits) {
     *waits = false;
+    std::lock_guard<std::mutex> lk(g_mem_mu);
     auto it = g_kept.find(dev);
     if (it == g_kept.end()) return nullptr;
     Kept &k = it->second;
@@ -102,28 +115,36 @@ void *take(int dev, size_t size, bool *waits) {
     return nullptr;
 }
 
-// (lock held) gives back everything kept on a device
+// gives back everything kept on a device (blocks that another thread is waiting for stay)
 void give_back(int dev) {
-    auto it = g_kept.find(dev);
-    if (it == g_kept.end()) return;
-    Kept &k = it->second;
-    for (auto &r : k.ready)
-        for (void *p : r.second) {
+    std::map<size_t, std::vector<void *>> ready;
+    std::vector<std::pair<size_t, void *>> waiting;
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lk(g_mem_mu);
+        auto it = g_kept.find(dev);
+        if (it == g_kept.end()) return;
+        Kept &k = it->second;
+        ready.swap(k.ready);
+        waiting.swap(k.waiting);
+        pool = k.pool;
+        auto unlist = [&](size_t size, void *p) {
+            k.bytes -= size;
             g_blocks.erase(p);
-            free_now(p);
-        }
-    for (const auto &w : k.waiting) {
-        g_blocks.erase(w.second);
-        free_now(w.second);
+        };
+        for (const auto &r : ready)
+            for (void *p : r.second) unlist(r.first, p);
+        for (const auto &w : waiting) unlist(w.first, w.second);
     }
-    k.ready.clear();
-    k.waiting.clear();
-    k.bytes = 0;
-    if (k.pool) cudaMemPoolTrimTo(k.pool, 0);
+    for (const auto &r : ready)
+        for (void *p : r.second) free_now(p);
+    for (const auto &w : waiting) free_now(w.second);
+    if (pool) cudaMemPoolTrimTo(pool, 0);
 }
 
-// (lock held) the library's pool of a device; null where it cannot be made
+// the library's pool of a device; null where it cannot be made
 cudaMemPool_t pool_of(int dev) {
+    std::lock_guard<std::mutex> lk(g_mem_mu);
     Kept &k = g_kept[dev];
     if (k.pool_tried) return k.pool;
     k.pool_tried = true;
@@ -151,7 +172,6 @@ cudaError_t dev_malloc(void **p, size_t bytes) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const size_t size = bytes <= SMALL_MOST ? block_size(bytes) : 0;
-    std::lock_guard<std::mutex> lk(g_mem_mu);
     if (size) {
         bool waits = false;
         *p = take(dev, size, &waits);
@@ -172,6 +192,7 @@ cudaError_t dev_malloc(void **p, size_t bytes) {
         return e;
     }
     if (size) try {
+            std::lock_guard<std::mutex> lk(g_mem_mu);
             g_blocks[*p] = Block{size, dev};
         } catch (const std::bad_alloc &) {  // unlisted: goes back at once when freed
         }
@@ -180,20 +201,22 @@ cudaError_t dev_malloc(void **p, size_t bytes) {
 
 void dev_free(void *p) {
     if (!p) return;
-    std::lock_guard<std::mutex> lk(g_mem_mu);
-    auto it = g_blocks.find(p);
-    if (it != g_blocks.end()) {
-        const Block b = it->second;
-        try {
-            Kept &k = g_kept[b.dev];
-            if (k.bytes + b.size <= SMALL_KEEP) {
-                k.waiting.emplace_back(b.size, p);
-                k.bytes += b.size;
-                return;
+    {
+        std::lock_guard<std::mutex> lk(g_mem_mu);
+        auto it = g_blocks.find(p);
+        if (it != g_blocks.end()) {
+            const Block b = it->second;
+            try {
+                Kept &k = g_kept[b.dev];
+                if (k.bytes + b.size <= SMALL_KEEP) {
+                    k.waiting.emplace_back(b.size, p);
+                    k.bytes += b.size;
+                    return;
+                }
+            } catch (const std::bad_alloc &) {
             }
-        } catch (const std::bad_alloc &) {
+            g_blocks.erase(it);  // before the address can be given out anew
         }
-        g_blocks.erase(it);
     }
     free_now(p);
 }
@@ -201,7 +224,6 @@ void dev_free(void *p) {
 void dev_settle() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return;
-    std::lock_guard<std::mutex> lk(g_mem_mu);
     settle(dev);
 }
 
@@ -211,19 +233,12 @@ cudaError_t dev_malloc_async(void **p, size_t bytes, cudaStream_t s) try {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    cudaMemPool_t pool;
-    {
-        std::lock_guard<std::mutex> lk(g_mem_mu);
-        pool = pool_of(dev);
-    }
+    cudaMemPool_t pool = pool_of(dev);
     if (!pool) return cudaMallocAsync(p, bytes, s);
     e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        {
-            std::lock_guard<std::mutex> lk(g_mem_mu);
-            give_back(dev);
-        }
+        give_back(dev);
         e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     }
     return e;

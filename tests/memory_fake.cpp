@@ -2,14 +2,30 @@
 // status 0 if it holds.  The fakes count, fail or block the calls they stand for.
 #include <cuda_runtime.h>
 
+#include <condition_variable>
 #include <cstdio>
 #include <map>
+#include <mutex>
 #include <set>
 #include <string>
+#include <thread>
 
 #include "memory.cuh"
 
 namespace {
+std::mutex g_mu;
+std::condition_variable g_cv;
+bool g_hold = false;          // cudaDeviceSynchronize and cudaFree block while set
+int g_held = 0;               // calls blocked
+
+void hold_point() {
+    std::unique_lock<std::mutex> lk(g_mu);
+    ++g_held;
+    g_cv.notify_all();
+    g_cv.wait(lk, [] { return !g_hold; });
+    --g_held;
+}
+
 std::set<void *> g_live;      // blocks of cudaMalloc not yet freed
 size_t g_next = 1 << 20;      // the next address
 int g_waits = 0, g_mallocs = 0;
@@ -33,6 +49,7 @@ extern "C" {
 cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }
 cudaError_t cudaMalloc(void **p, size_t n) {
+    std::lock_guard<std::mutex> lk(g_mu);
     ++g_mallocs;
     *p = reinterpret_cast<void *>(g_next);
     g_next += (n + 255) / 256 * 256;
@@ -41,9 +58,12 @@ cudaError_t cudaMalloc(void **p, size_t n) {
 }
 cudaError_t cudaFree(void *p) {
     if (!p) return cudaSuccess;
+    hold_point();
+    std::lock_guard<std::mutex> lk(g_mu);
     return g_live.erase(p) ? cudaSuccess : cudaErrorInvalidValue;
 }
 cudaError_t cudaDeviceSynchronize(void) {
+    hold_point();
     ++g_waits;
     return g_wait_status;
 }
@@ -96,8 +116,38 @@ static int bounded() {
     return 0;
 }
 
+// a thread that waits for the device, or frees a large block, holds up nobody else
+static int threads() {
+    void *a = get(5000), *big = get(size_t(9) << 20), *b = get(700);
+    for (int round = 0; round < 2; ++round) {
+        g_hold = true;
+        std::thread t(round == 0 ? [](void *small, void *) { spmv::dev_free(small), spmv::dev_settle(); }
+                                 : [](void *, void *large) { spmv::dev_free(large); },
+                      a, big);
+        {
+            std::unique_lock<std::mutex> lk(g_mu);
+            g_cv.wait(lk, [] { return g_held == 1; });
+        }
+        void *c = get(9000 << round);  // (blocks for good where the lock is held: the run is then ended from outside)
+        CHECK(c && c != a);
+        spmv::dev_free(c);
+        if (round == 0) spmv::dev_free(b);  // freed after the wait began: not ready when it ends
+        {
+            std::lock_guard<std::mutex> lk(g_mu);
+            g_hold = false;
+        }
+        g_cv.notify_all();
+        t.join();
+    }
+    const int waits = g_waits;
+    CHECK(get(5000) == a && g_waits == waits);
+    CHECK(get(700) == b && g_waits == waits + 1);
+    return 0;
+}
+
 int main(int argc, char **argv) {
-    const std::map<std::string, int (*)()> all = {{"reuse", reuse}, {"failed_wait", failed_wait}, {"bounded", bounded}};
+    const std::map<std::string, int (*)()> all = {{"reuse", reuse}, {"failed_wait", failed_wait}, {"bounded", bounded},
+                                                       {"threads", threads}};
     const auto it = all.find(argc > 1 ? argv[1] : "");
     return it == all.end() ? 2 : it->second();
 }
