@@ -10,7 +10,15 @@
 // synchronisations (the default pool unmaps at each: 2 us per MB to map and
 // unmap).  At most SMALL_KEEP + POOL_KEEP bytes are kept per device (0.1% of
 // it); what exceeds them goes back at once, the rest when an allocation fails.
+//
+// Blocks and pool belong to a context, not to a device: cudaDeviceReset ends
+// the context and with it everything kept, and a context of the driver API has
+// memory of its own.  The tables go by the id of the context, which the driver
+// never gives twice; what belonged to a context that has ended is not touched
+// again, not even freed (its addresses may be someone else's by then).
 #include "memory.cuh"
+
+#include <cuda.h>
 
 #include <cstdint>
 #include <cstdlib>
@@ -38,11 +46,15 @@ bool fault_injected() {
 
 constexpr size_t SMALL_MOST = size_t(8) << 20, SMALL_KEEP = size_t(64) << 20, POOL_KEEP = size_t(256) << 20;
 
-struct Block {
-    size_t size;
-    int dev;
+struct Context {
+    CUcontext handle = nullptr;
+    uint64_t id = 0;  // 0: none to be had; nothing is kept then
 };
-// what is kept of one device
+struct Block {
+    size_t size;  // 0: larger than SMALL_MOST, not kept
+    Context ctx;
+};
+// what is kept of one context
 struct Kept {
     std::map<size_t, std::vector<void *>> ready;      // idle blocks by size
     std::vector<std::pair<size_t, void *>> waiting;   // freed since the device was last waited for
@@ -51,8 +63,35 @@ struct Kept {
     bool pool_tried = false;
 };
 std::mutex g_mem_mu;  // guards the tables; not held while the device is waited for or memory mapped
-std::unordered_map<void *, Block> g_blocks;  // every small block handed out or kept
-std::map<int, Kept> g_kept;                  // by device
+std::unordered_map<void *, Block> g_blocks;  // every block handed out or kept
+std::map<uint64_t, Kept> g_kept;             // by context
+
+template <typename F>
+F driver(const char *name) {
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion(name, &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return reinterpret_cast<F>(fn);
+}
+
+// id of a context; 0 if it has ended
+uint64_t id_of(CUcontext handle) {
+    static const auto get = driver<CUresult (*)(CUcontext, unsigned long long *)>("cuCtxGetId");
+    unsigned long long id = 0;
+    return get && handle && get(handle, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+Context current_context() {
+    static const auto get = driver<CUresult (*)(CUcontext *)>("cuCtxGetCurrent");
+    Context c;
+    if (cudaFree(nullptr) != cudaSuccess) cudaGetLastError();  // (makes the device's context if there is none)
+    else if (get && get(&c.handle) == CUDA_SUCCESS) c.id = id_of(c.handle);
+    return c;
+}
 
 // four sizes an octave: at most a quarter more than asked for
 size_t block_size(size_t bytes) {
@@ -71,11 +110,11 @@ void free_now(void *p) {
 }
 
 // waits for the device, then makes the blocks freed before the wait ready
-void settle(int dev) {
+void settle(uint64_t ctx) {
     std::vector<std::pair<size_t, void *>> w;
     {
         std::lock_guard<std::mutex> lk(g_mem_mu);
-        auto it = g_kept.find(dev);
+        auto it = g_kept.find(ctx);
         if (it == g_kept.end() || it->second.waiting.empty()) return;
         w.swap(it->second.waiting);
     }
@@ -84,7 +123,7 @@ void settle(int dev) {
     size_t left = 0;  // blocks the host has no memory to list: they go back
     {
         std::lock_guard<std::mutex> lk(g_mem_mu);
-        Kept &k = g_kept.find(dev)->second;
+        Kept &k = g_kept.find(ctx)->second;
         for (const auto &b : w) try {
                 if (idle) k.ready[b.first].push_back(b.second);
                 else k.waiting.push_back(b);
@@ -98,10 +137,10 @@ void settle(int dev) {
 }
 
 // a ready block of the size, or null; *waits: blocks of the size are waiting
-void *take(int dev, size_t size, bool *waits) {
+void *take(uint64_t ctx, size_t size, bool *waits) {
     *waits = false;
     std::lock_guard<std::mutex> lk(g_mem_mu);
-    auto it = g_kept.find(dev);
+    auto it = g_kept.find(ctx);
     if (it == g_kept.end()) return nullptr;
     Kept &k = it->second;
     auto r = k.ready.find(size);
@@ -115,14 +154,14 @@ void *take(int dev, size_t size, bool *waits) {
     return nullptr;
 }
 
-// gives back everything kept on a device (blocks that another thread is waiting for stay)
-void give_back(int dev) {
+// gives back everything kept of the current context (blocks that another thread is waiting for stay)
+void give_back(uint64_t ctx) {
     std::map<size_t, std::vector<void *>> ready;
     std::vector<std::pair<size_t, void *>> waiting;
     cudaMemPool_t pool;
     {
         std::lock_guard<std::mutex> lk(g_mem_mu);
-        auto it = g_kept.find(dev);
+        auto it = g_kept.find(ctx);
         if (it == g_kept.end()) return;
         Kept &k = it->second;
         ready.swap(k.ready);
@@ -142,10 +181,12 @@ void give_back(int dev) {
     if (pool) cudaMemPoolTrimTo(pool, 0);
 }
 
-// the library's pool of a device; null where it cannot be made
-cudaMemPool_t pool_of(int dev) {
+// the library's pool of the current context; null where it cannot be made
+cudaMemPool_t pool_of(uint64_t ctx) {
+    int dev = 0;
+    if (!ctx || cudaGetDevice(&dev) != cudaSuccess) return nullptr;
     std::lock_guard<std::mutex> lk(g_mem_mu);
-    Kept &k = g_kept[dev];
+    Kept &k = g_kept[ctx];
     if (k.pool_tried) return k.pool;
     k.pool_tried = true;
     cudaMemPoolProps props{};
@@ -168,32 +209,31 @@ void reset_alloc_count() { g_alloc_count = 0; }
 cudaError_t dev_malloc(void **p, size_t bytes) {
     *p = nullptr;
     if (fault_injected()) return cudaErrorMemoryAllocation;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const size_t size = bytes <= SMALL_MOST ? block_size(bytes) : 0;
+    const Context c = current_context();
+    const uint64_t ctx = c.id;
+    const size_t size = ctx && bytes <= SMALL_MOST ? block_size(bytes) : 0;
     if (size) {
         bool waits = false;
-        *p = take(dev, size, &waits);
+        *p = take(ctx, size, &waits);
         if (!*p && waits) {
-            settle(dev);
-            *p = take(dev, size, &waits);
+            settle(ctx);
+            *p = take(ctx, size, &waits);
         }
         if (*p) return cudaSuccess;
     }
-    e = cudaMalloc(p, size ? size : bytes);
+    cudaError_t e = cudaMalloc(p, size ? size : bytes);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        give_back(dev);
+        give_back(ctx);
         e = cudaMalloc(p, size ? size : bytes);
     }
     if (e != cudaSuccess) {
         *p = nullptr;
         return e;
     }
-    if (size) try {
+    if (ctx) try {
             std::lock_guard<std::mutex> lk(g_mem_mu);
-            g_blocks[*p] = Block{size, dev};
+            g_blocks[*p] = Block{size, c};
         } catch (const std::bad_alloc &) {  // unlisted: goes back at once when freed
         }
     return e;
@@ -201,13 +241,18 @@ cudaError_t dev_malloc(void **p, size_t bytes) {
 
 void dev_free(void *p) {
     if (!p) return;
+    const uint64_t ctx = current_context().id;
     {
         std::lock_guard<std::mutex> lk(g_mem_mu);
         auto it = g_blocks.find(p);
         if (it != g_blocks.end()) {
             const Block b = it->second;
-            try {
-                Kept &k = g_kept[b.dev];
+            if (ctx != b.ctx.id && id_of(b.ctx.handle) != b.ctx.id) {
+                g_blocks.erase(it);
+                return;
+            }
+            if (b.size && ctx == b.ctx.id) try {
+                Kept &k = g_kept[ctx];
                 if (k.bytes + b.size <= SMALL_KEEP) {
                     k.waiting.emplace_back(b.size, p);
                     k.bytes += b.size;
@@ -221,24 +266,18 @@ void dev_free(void *p) {
     free_now(p);
 }
 
-void dev_settle() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return;
-    settle(dev);
-}
+void dev_settle() { settle(current_context().id); }
 
 cudaError_t dev_malloc_async(void **p, size_t bytes, cudaStream_t s) try {
     *p = nullptr;
     if (fault_injected()) return cudaErrorMemoryAllocation;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    cudaMemPool_t pool = pool_of(dev);
+    const uint64_t ctx = current_context().id;
+    cudaMemPool_t pool = pool_of(ctx);
     if (!pool) return cudaMallocAsync(p, bytes, s);
-    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        give_back(dev);
+        give_back(ctx);
         e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     }
     return e;

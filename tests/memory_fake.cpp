@@ -1,9 +1,11 @@
 // memory.cu against a fake CUDA runtime: one scenario a run (argv[1]), exit
 // status 0 if it holds.  The fakes count, fail or block the calls they stand for.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <condition_variable>
 #include <cstdio>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <set>
@@ -30,6 +32,18 @@ std::set<void *> g_live;      // blocks of cudaMalloc not yet freed
 size_t g_next = 1 << 20;      // the next address
 int g_waits = 0, g_mallocs = 0;
 cudaError_t g_wait_status = cudaSuccess;
+unsigned long long g_context = 1;  // the current context's id
+std::set<size_t> g_pools_used;     // pools temporaries came from
+size_t g_pools = 0;
+
+CUresult current(CUcontext *c) {
+    *c = reinterpret_cast<CUcontext>(0x100);
+    return CUDA_SUCCESS;
+}
+CUresult context_id(CUcontext, unsigned long long *id) {
+    *id = g_context;
+    return CUDA_SUCCESS;
+}
 
 #define CHECK(c)                                               \
     do {                                                       \
@@ -67,11 +81,24 @@ cudaError_t cudaDeviceSynchronize(void) {
     ++g_waits;
     return g_wait_status;
 }
-cudaError_t cudaMemPoolCreate(cudaMemPool_t *, const cudaMemPoolProps *) { return cudaErrorNotSupported; }
+cudaError_t cudaMemPoolCreate(cudaMemPool_t *p, const cudaMemPoolProps *) {
+    *p = reinterpret_cast<cudaMemPool_t>(++g_pools);
+    return cudaSuccess;
+}
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }
 cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t) { return cudaSuccess; }
-cudaError_t cudaMallocFromPoolAsync(void **, size_t, cudaMemPool_t, cudaStream_t) { return cudaErrorNotSupported; }
+cudaError_t cudaMallocFromPoolAsync(void **p, size_t, cudaMemPool_t pool, cudaStream_t) {
+    g_pools_used.insert(reinterpret_cast<size_t>(pool));
+    *p = &g_pools_used;
+    return cudaSuccess;
+}
 cudaError_t cudaMallocAsync(void **, size_t, cudaStream_t) { return cudaErrorNotSupported; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char *name, void **fn, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult *found) {
+    *fn = !std::strcmp(name, "cuCtxGetId") ? reinterpret_cast<void *>(&context_id) : reinterpret_cast<void *>(&current);
+    *found = cudaDriverEntryPointSuccess;
+    return cudaSuccess;
+}
 }
 
 // a freed block is handed out again after a wait that succeeded, not before
@@ -145,9 +172,35 @@ static int threads() {
     return 0;
 }
 
+// a device reset ends the context: nothing of it is handed out, used or listed
+// again, nor freed, since its addresses are given anew
+static int reset() {
+    void *a = get(5000), *b = get(6000), *c = get(7000), *big = get(size_t(9) << 20), *t = nullptr;
+    spmv::dev_free(a);
+    spmv::dev_settle();
+    spmv::dev_free(b);
+    CHECK(spmv::dev_malloc_async(&t, 100, nullptr) == cudaSuccess);
+    g_context = 2;
+    const std::set<void *> others = g_live;  // somebody else's blocks in the new context
+    CHECK(get(5000) != a && get(6000) != b && g_mallocs == 6);
+    spmv::dev_free(c);  // of the old context
+    spmv::dev_free(big);
+    for (void *p : others) CHECK(g_live.count(p));
+    CHECK(get(7000) != c);
+    spmv::dev_settle();
+    CHECK(get(7000) != c);
+    CHECK(spmv::dev_malloc_async(&t, 100, nullptr) == cudaSuccess);
+    CHECK(g_pools == 2 && g_pools_used == (std::set<size_t>{1, 2}));
+    void *d = get(5000);  // the new one keeps its own
+    spmv::dev_free(d);
+    spmv::dev_settle();
+    CHECK(get(5000) == d);
+    return 0;
+}
+
 int main(int argc, char **argv) {
     const std::map<std::string, int (*)()> all = {{"reuse", reuse}, {"failed_wait", failed_wait}, {"bounded", bounded},
-                                                       {"threads", threads}};
+                                                       {"threads", threads},   {"reset", reset}};
     const auto it = all.find(argc > 1 ? argv[1] : "");
     return it == all.end() ? 2 : it->second();
 }

@@ -1,6 +1,7 @@
 """The library's device memory (csrc/memory.cu) against a fake CUDA runtime
 (memory_fake.cpp), on the host: when a freed block is handed out again,
-how much is kept, and that threads do not wait for each other's frees."""
+how much is kept, that threads do not wait for each other's frees,
+and that nothing kept outlives its context."""
 import os
 import shutil
 import subprocess
@@ -21,7 +22,7 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("scenario", ["reuse", "failed_wait", "bounded", "threads"])
+@pytest.mark.parametrize("scenario", ["reuse", "failed_wait", "bounded", "threads", "reset"])
 def test_scenario(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=20)
     assert r.returncode == 0, r.stdout
