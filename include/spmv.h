@@ -563,8 +563,23 @@ SPMV_API int64_t spmv_get_panel_limit(void);
  */
 SPMV_API int spmv_check(spmv_handle h, void *stream);
 
-/* Frees every device array of the handle.  NULL is accepted. */
+/*
+ * Frees every device array of the handle, after the work launched on the
+ * device is done.  NULL is accepted.  Arrays of up to 8 MiB are kept for later
+ * calls (spmv_trim).
+ */
 SPMV_API int spmv_destroy(spmv_handle h);
+
+/*
+ * Device memory the library keeps (no counterpart in the paper).  Mapping and
+ * unmapping device memory takes longer than many of the library's calls, so
+ * freed arrays of up to 8 MiB (at most 64 MiB of them) and the memory of the
+ * calls' temporaries (at most 256 MiB) are kept for later calls, per device.
+ * They go back when an allocation of the library fails; spmv_trim gives them
+ * back at once, for callers whose other libraries need the memory, on the
+ * current device.  Waits for the device's work.  Errors: SPMV_ERR_CUDA.
+ */
+SPMV_API int spmv_trim(void);
 
 /* Message of the last failing call on this thread ("" if none). */
 SPMV_API const char *spmv_last_error(void);

@@ -721,6 +721,12 @@ int spmv_check(spmv_handle h, void *stream) {
     return SPMV_OK;
 }
 
+int spmv_trim(void) {
+    entry_reset();
+    SPMV_CUDA_TRY(dev_trim());
+    return SPMV_OK;
+}
+
 int spmv_destroy(spmv_handle h) {
     if (!h) return SPMV_OK;
     destroy_all(h);

@@ -9,7 +9,8 @@
 // pool of the library that keeps POOL_KEEP bytes mapped across the call's own
 // synchronisations (the default pool unmaps at each: 2 us per MB to map and
 // unmap).  At most SMALL_KEEP + POOL_KEEP bytes are kept per device (0.1% of
-// it); what exceeds them goes back at once, the rest when an allocation fails.
+// it); what exceeds them goes back at once, the rest when an allocation fails or
+// the caller asks for it (spmv_trim).
 //
 // Blocks and pool belong to a context, not to a device: cudaDeviceReset ends
 // the context and with it everything kept, and a context of the driver API has
@@ -264,6 +265,13 @@ void dev_free(void *p) {
         }
     }
     free_now(p);
+}
+
+cudaError_t dev_trim() {
+    const uint64_t ctx = current_context().id;
+    const cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) give_back(ctx);
+    return e;
 }
 
 void dev_settle() { settle(current_context().id); }

@@ -28,5 +28,7 @@ void reset_alloc_count();
 void dev_free(void *p);
 // Waits for the device's work; blocks freed before are then handed out again.
 void dev_settle();
+// Gives back what is kept of the current context, after the device's work is done.
+cudaError_t dev_trim();
 
 }  // namespace spmv

@@ -34,7 +34,7 @@ int g_waits = 0, g_mallocs = 0;
 cudaError_t g_wait_status = cudaSuccess;
 unsigned long long g_context = 1;  // the current context's id
 std::set<size_t> g_pools_used;     // pools temporaries came from
-size_t g_pools = 0;
+size_t g_pools = 0, g_trims = 0;
 
 CUresult current(CUcontext *c) {
     *c = reinterpret_cast<CUcontext>(0x100);
@@ -86,7 +86,10 @@ cudaError_t cudaMemPoolCreate(cudaMemPool_t *p, const cudaMemPoolProps *) {
     return cudaSuccess;
 }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }
-cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t) { return cudaSuccess; }
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t keep) {
+    g_trims += keep == 0;
+    return cudaSuccess;
+}
 cudaError_t cudaMallocFromPoolAsync(void **p, size_t, cudaMemPool_t pool, cudaStream_t) {
     g_pools_used.insert(reinterpret_cast<size_t>(pool));
     *p = &g_pools_used;
@@ -198,9 +201,27 @@ static int reset() {
     return 0;
 }
 
+// everything kept can be given back
+static int trim() {
+    void *a = get(5000), *b = get(6000), *c = get(7000), *t = nullptr;
+    CHECK(spmv::dev_malloc_async(&t, 100, nullptr) == cudaSuccess);
+    spmv::dev_free(a);
+    spmv::dev_settle();
+    spmv::dev_free(b);
+    g_wait_status = cudaErrorStreamCaptureUnsupported;
+    CHECK(spmv::dev_trim() != cudaSuccess && g_live.size() == 3);
+    g_wait_status = cudaSuccess;
+    CHECK(spmv::dev_trim() == cudaSuccess);
+    CHECK(g_live == std::set<void *>{c} && g_trims == 1);
+    spmv::dev_free(c);
+    CHECK(spmv::dev_trim() == cudaSuccess && g_live.empty());
+    return 0;
+}
+
 int main(int argc, char **argv) {
     const std::map<std::string, int (*)()> all = {{"reuse", reuse}, {"failed_wait", failed_wait}, {"bounded", bounded},
-                                                       {"threads", threads},   {"reset", reset}};
+                                                       {"threads", threads},   {"reset", reset},
+                                                       {"trim", trim}};
     const auto it = all.find(argc > 1 ? argv[1] : "");
     return it == all.end() ? 2 : it->second();
 }

@@ -1,7 +1,7 @@
 """The library's device memory (csrc/memory.cu) against a fake CUDA runtime
 (memory_fake.cpp), on the host: when a freed block is handed out again,
 how much is kept, that threads do not wait for each other's frees,
-and that nothing kept outlives its context."""
+that nothing kept outlives its context, and that it can be given back."""
 import os
 import shutil
 import subprocess
@@ -22,7 +22,7 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("scenario", ["reuse", "failed_wait", "bounded", "threads", "reset"])
+@pytest.mark.parametrize("scenario", ["reuse", "failed_wait", "bounded", "threads", "reset", "trim"])
 def test_scenario(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=20)
     assert r.returncode == 0, r.stdout
