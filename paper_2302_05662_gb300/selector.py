@@ -31,14 +31,17 @@ LOWP_BLOB = os.path.join(PKG, "selector_gb300_fp32_values.f32")
 BF16_BLOB = os.path.join(PKG, "selector_gb300_bf16_values.f32")
 # the exhaustive-sweep records the committed fp64 selector was trained on
 # (every label point of the 2000 dataset matrices, L2 flushed by reading,
-# trimmed means), the conversion-time calibration of its cost model, and the
-# GPU-measured held-out evaluations (sweep --heldout-eval) of the fp64, fp32 and
-# bf16 selectors
+# trimmed means), and the GPU-measured held-out evaluations (sweep
+# --heldout-eval) of the fp64, fp32 and bf16 selectors
 DEFAULT_DATA = os.path.join(PKG, "data", "sweep_gb300_f64_readflush.jsonl.gz")
-DEFAULT_CALIB = os.path.join(PKG, "data", "convert_calib_gb300_f64.jsonl.gz")
 RETIMED_F64 = os.path.join(PKG, "data", "heldout_retimed_gb300_f64.jsonl.gz")
 RETIMED_F32 = os.path.join(PKG, "data", "heldout_retimed_gb300_f32.jsonl.gz")
 RETIMED_BF16 = os.path.join(PKG, "data", "heldout_retimed_gb300_bf16.jsonl.gz")
+# sweeps of the same matrices and configurations on the kernels as they are
+# now, and conversion times of each value type: what the time heads and the
+# conversion-cost lines of the blobs (the run-time gate) are fitted to
+HEADS_DATA = {vt: os.path.join(PKG, "data", f"heads_gb300_{vt}.jsonl.gz") for vt in ("f64", "f32", "bf16")}
+HEADS_CALIB = os.path.join(PKG, "data", "heads_convert_gb300.jsonl.gz")
 MAGIC, VERSION = 2302.0, 1.0
 CFG_FIELDS = ("format", "threads_per_block", "threads_per_row", "unroll", "regcap", "carveout",
               "bsr_block", "hyb_ell_width")
@@ -432,11 +435,71 @@ def evaluate_retimed(paths) -> dict:
     return out
 
 
+def fit_heads(w, recs, calib, labels, holdout_start: int = 1800):
+    """The blob's time head and conversion-cost lines, fitted to the records
+    and conversion times of matrices below holdout_start, and their report on
+    the others: what the classifier's choice reaches there, the head's errors,
+    the lines' errors, and how often the gate decides as the measured times
+    would.  Returns (W3, b3, pack, report)."""
+    from . import sweep
+    X, T, D, ids, fams = dataset(recs, [sweep.config_key(c) for c in labels])
+    ok = np.isfinite(T).any(axis=1) & np.isfinite(D)
+    train_m, test_m = ok & (ids < holdout_start), ok & (ids >= holdout_start)
+    W3, b3 = train_time_head(w, X[train_m], T[train_m], D[train_m])
+    pack = fit_pack_model([c for c in calib if c["matrix"] < holdout_start])
+    report = {"pack_model_us": {str(f): [float(v) for v in pack[f]] for f in range(NFMT)}}
+    if not test_m.any():
+        return W3, b3, pack, report
+    lt = predict_logt(w, W3, b3, X[test_m])
+    choice = np.argmax(np.where(np.isfinite(T[test_m]), predict(w, X[test_m]), -np.inf), axis=1)
+    rows = np.arange(choice.size)
+    report["heldout"] = evaluate(choice, T[test_m], D[test_m])
+    fam = np.array(fams)[test_m]
+    report["heldout_by_family"] = {f: evaluate(choice[fam == f], T[test_m][fam == f], D[test_m][fam == f])
+                                   for f in sorted(set(fam))}
+    # error of the selected class and of default CSR
+    e_sel = np.abs(lt[rows, choice] - np.log(T[test_m][rows, choice]))
+    e_def = np.abs(lt[:, -1] - np.log(D[test_m]))
+    report["time_head_heldout"] = {"median_abs_log_error_selected": float(np.median(e_sel)),
+                                   "median_abs_log_error_default_csr": float(np.median(e_def)),
+                                   "p90_abs_log_error_selected": float(np.quantile(e_sel, 0.9)),
+                                   "p90_abs_log_error_default_csr": float(np.quantile(e_def, 0.9))}
+    held = [c for c in calib if c["matrix"] >= holdout_start and c["us"] is not None]
+    if not held:
+        return W3, b3, pack, report
+    pred = np.array([pack[c["format"]] @ [1.0, c["nnz"], c["m"]] for c in held])
+    meas = np.array([c["us"] for c in held])
+    report["pack_model_heldout"] = {"n": len(held),
+                                    "r2": 1.0 - float(((pred - meas) ** 2).sum() / ((meas - meas.mean()) ** 2).sum()),
+                                    "median_abs_rel_error": float(np.median(np.abs(pred - meas) / meas))}
+    # the gate: predicted vs measured decision
+    by = {}
+    for c in held:
+        by.setdefault(c["matrix"], {})[c["format"]] = c
+    agree = {}
+    for runs in (1, 10, 100, 1000, 10000):
+        hits = []
+        for i, mid in enumerate(ids[test_m]):
+            f = int(labels[choice[i]]["format"])
+            c = by.get(mid, {}).get(f)
+            if c is None:
+                continue
+            truth = gate_decision(D[test_m][i], T[test_m][i, choice[i]], 0.0, c["us"], runs)
+            guess = gate_decision(np.exp(lt[i, -1]), np.exp(lt[i, choice[i]]), 0.0, pack[f] @ [1.0, c["nnz"], c["m"]], runs)
+            hits.append(truth == guess)
+        agree[str(runs)] = float(np.mean(hits)) if hits else None
+    report["gate_agreement_heldout"] = agree
+    return W3, b3, pack, report
+
+
 def main():
     """Train on the sweep records (matrices 0-1799), evaluate on 1800-1999,
     write the blob and a JSON report.  With --calib (conversion-time
     records) the blob is version 2: time head + conversion-cost model, and
-    the report evaluates the run-time gate on the held-out matrices."""
+    the report evaluates the run-time gate on the held-out matrices.  With
+    --heads-data both come from a later sweep than the classifier's labels,
+    and the report's "classifier_on_heads_data" says what its choice reaches
+    there."""
     import argparse
     from . import sweep
     ap = argparse.ArgumentParser(description="train the selector MLP from sweep records")
@@ -448,6 +511,9 @@ def main():
     ap.add_argument("--holdout-start", type=int, default=1800)
     ap.add_argument("--from-blob", default=None, help="reuse this blob's classifier, fit only the heads")
     ap.add_argument("--calib", nargs="*", default=None, help="conversion-time records (JSON lines)")
+    ap.add_argument("--heads-data", nargs="*", default=None,
+                    help="sweep records that the time head is fitted to (default: those of --data)")
+    ap.add_argument("--calib-dtype", default=None, help="use only the conversion-time records of this value type")
     ap.add_argument("--refine", nargs="*", default=None,
                     help="refine records (sweep --refine-from): evaluate a per-class register cap / unroll / "
                          "carveout table against the refined exhaustive best")
@@ -488,53 +554,13 @@ def main():
         for path in args.calib:
             with (gzip.open(path, "rt") if path.endswith(".gz") else open(path)) as fh:
                 calib += [json.loads(l) for l in fh if l.strip()]
-        W3, b3 = train_time_head(w, X[train_m], T[train_m], D[train_m])
-        pack = fit_pack_model([c for c in calib if c["matrix"] < args.holdout_start])
-        # time head on held-out matrices: error of the selected class and default CSR
-        if not test_m.any():   # no held-out sweep records (evaluated by --heldout-retimed instead)
-            test_m = train_m & False
-        lt = predict_logt(w, W3, b3, X[test_m]) if test_m.any() else None
-        if lt is not None:
-            logits = np.where(np.isfinite(T[test_m]), predict(w, X[test_m]), -np.inf)
-            choice = np.argmax(logits, axis=1)
-            rows = np.arange(choice.size)
-            e_sel = np.abs(lt[rows, choice] - np.log(T[test_m][rows, choice]))
-            e_def = np.abs(lt[:, -1] - np.log(D[test_m]))
-            report["time_head_heldout"] = {"median_abs_log_error_selected": float(np.median(e_sel)),
-                                           "median_abs_log_error_default_csr": float(np.median(e_def)),
-                                           "p90_abs_log_error_selected": float(np.quantile(e_sel, 0.9))}
-        # conversion-cost model on held-out calibration records
-        held = [c for c in calib if c["matrix"] >= args.holdout_start and c["us"] is not None]
-        if held and lt is not None:
-            pred = np.array([pack[c["format"]] @ [1.0, c["nnz"], c["m"]] for c in held])
-            meas = np.array([c["us"] for c in held])
-            ss_res = float(((pred - meas) ** 2).sum())
-            ss_tot = float(((meas - meas.mean()) ** 2).sum())
-            report["pack_model_heldout"] = {"n": len(held), "r2": 1.0 - ss_res / ss_tot,
-                                            "median_abs_rel_error": float(np.median(np.abs(pred - meas) / meas))}
-            # the gate on held-out matrices: predicted vs measured decision
-            by = {}
-            for c in held:
-                by.setdefault(c["matrix"], {})[c["format"]] = c["us"]
-            id_test = ids[test_m]
-            agree = {}
-            for runs in (1, 10, 100, 1000, 10000):
-                hits = tot = 0
-                for i, mid in enumerate(id_test):
-                    if mid not in by:
-                        continue
-                    f = int(labels[choice[i]]["format"])
-                    if f not in by[mid]:
-                        continue
-                    t_def, t_sel = D[test_m][i], T[test_m][i, choice[i]]
-                    truth = gate_decision(t_def, t_sel, 0.0, by[mid][f], runs)
-                    guess = gate_decision(np.exp(lt[i, -1]), np.exp(lt[i, choice[i]]), 0.0,
-                                          pack[f] @ [1.0, by_nnz(recs, mid), by_m(recs, mid)], runs)
-                    hits += int(truth == guess)
-                    tot += 1
-                agree[str(runs)] = hits / tot if tot else None
-            report["gate_agreement_heldout"] = agree
-        report["pack_model_us"] = {str(f): [float(v) for v in pack[f]] for f in range(NFMT)}
+        if args.calib_dtype:
+            calib = [c for c in calib if c["dtype"] == args.calib_dtype]
+        heads = load_records(args.heads_data) if args.heads_data else recs
+        W3, b3, pack, found = fit_heads(w, heads, calib, labels, args.holdout_start)
+        report.update({k: v for k, v in found.items() if not k.startswith("heldout")})
+        if args.heads_data:
+            report["classifier_on_heads_data"] = {k: v for k, v in found.items() if k.startswith("heldout")}
     if args.refine:
         refine = load_refine(args.refine)
         table = knob_table(refine, ids[train_m])
@@ -557,14 +583,6 @@ def main():
         with open(args.report, "w") as fh:
             fh.write(txt + "\n")
     print(txt)
-
-
-def by_nnz(recs, mid):
-    return next(r["nnz"] for r in recs if r["matrix"] == mid)
-
-
-def by_m(recs, mid):
-    return next(r["m"] for r in recs if r["matrix"] == mid)
 
 
 if __name__ == "__main__":

@@ -209,40 +209,46 @@ def generate_dataset_matrix(idx: int, n_lo=1e3, n_hi=2.1e6):
     return fam, matgen.family_matrix(fam, n, seed=20_000 + idx, jitter=True)
 
 
-def calibrate_pack(indices, out_path, reps: int = 3):
-    """Conversion-cost calibration: for dataset matrices `indices`, the wall
-    time of spmv_set_config from default CSR to each format (CSR as the
-    split variant), median of `reps`.  Appends JSON lines {matrix, format,
-    nnz, m, us}."""
+def calibrate_matrix(idx, fam, coo, reps: int = 3, value_dtype: str = "f64") -> list:
+    """Conversion-cost calibration of one matrix: the wall time of
+    spmv_set_config from default CSR to each format (CSR as the split
+    variant), median of `reps`, as records {matrix, dtype, format, nnz, m, us}."""
     import torch
+    rows, cols, vals = device_matrix(coo, value_dtype)
+    h = B.spmv_create(coo.m, coo.n, rows, cols, vals)
+    del rows, cols, vals
+    out = []
+    try:
+        for f in range(6):
+            cfg = dict(format=f)
+            if f == B.FMT_CSR:
+                cfg["threads_per_row"] = B.TPR_SPLIT
+            ts = []
+            for _ in range(reps):
+                B.spmv_set_config(h, B.make_config(format=B.FMT_CSR))
+                torch.cuda.synchronize()
+                t0 = time.perf_counter()
+                try:
+                    B.spmv_set_config(h, B.make_config(**cfg))
+                except B.SpmvError:
+                    ts = None
+                    break
+                ts.append((time.perf_counter() - t0) * 1e6)
+            out.append({"matrix": idx, "family": fam, "dtype": value_dtype, "format": f, "nnz": coo.nnz, "m": coo.m,
+                        "us": round(statistics.median(ts), 1) if ts else None})
+    finally:
+        B.spmv_destroy(h)
+    return out
+
+
+def calibrate_pack(indices, out_path, reps: int = 3, value_dtype: str = "f64"):
+    """calibrate_matrix for dataset matrices `indices`; appends JSON lines."""
     with open(out_path, "a") as fh:
         for idx in indices:
             fam, coo = generate_dataset_matrix(idx)
-            rows, cols, vals = device_matrix(coo)
-            h = B.spmv_create(coo.m, coo.n, rows, cols, vals)
-            del rows, cols, vals
-            try:
-                for f in range(6):
-                    cfg = dict(format=f)
-                    if f == B.FMT_CSR:
-                        cfg["threads_per_row"] = B.TPR_SPLIT
-                    ts = []
-                    for _ in range(reps):
-                        B.spmv_set_config(h, B.make_config(format=B.FMT_CSR))
-                        torch.cuda.synchronize()
-                        t0 = time.perf_counter()
-                        try:
-                            B.spmv_set_config(h, B.make_config(**cfg))
-                        except B.SpmvError:
-                            ts = None
-                            break
-                        ts.append((time.perf_counter() - t0) * 1e6)
-                    us = statistics.median(ts) if ts else None
-                    fh.write(json.dumps({"matrix": idx, "family": fam, "format": f, "nnz": coo.nnz, "m": coo.m,
-                                         "us": us}) + "\n")
-                fh.flush()
-            finally:
-                B.spmv_destroy(h)
+            for r in calibrate_matrix(idx, fam, coo, reps, value_dtype):
+                fh.write(json.dumps(r) + "\n")
+            fh.flush()
 
 
 def best_label(records_by_matrix: dict, idx: int):
@@ -437,7 +443,7 @@ def main():
         refine_sweep(args, Timer(flush=args.flush, stat=args.stat))
         return
     if args.calibrate_pack:
-        calibrate_pack(range(args.start, args.start + args.count), args.out)
+        calibrate_pack(range(args.start, args.start + args.count), args.out, value_dtype=args.dtype)
         return
     done = set()
     if os.path.exists(args.out):
