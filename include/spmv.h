@@ -407,16 +407,17 @@ SPMV_API int spmv_select(spmv_handle h, spmv_config *out_cfg, double *h_features
  * beta_i y_i in one persistent launch).  The paper runs one kernel per
  * matrix; a batch of hundreds of uneven matrices would then pay one launch
  * each.  A batch plan holds, for every matrix, a mode and a list of warp
- * work items over all matrices that a grid of resident thread blocks
- * consumes through one atomic counter.  A matrix whose handle holds ELL or
- * SELL runs in that format (ELL: 32 rows per item, a row per lane; SELL:
- * the handle's work items; mode -1 and -5), a COO handle as COO chunks of
- * 32*items entries per warp (mode -2) and a BSR handle as groups of 32 / r
- * block rows with r lanes each (mode -4), unless the tuner finds a CSR mode
- * faster; any other handle runs from its CSR arrays as nonzero chunks of
- * 32*items entries per warp (split, mode 0) or 32-row groups with 1..32
- * lanes per row (vector, mode = lanes per row).
- * The counter reset and the kernel are captured in a CUDA graph.
+ * work items over all matrices (about 1024 entries each) that a grid of
+ * resident thread blocks consumes through one atomic counter.  A matrix whose
+ * handle holds ELL or SELL runs in that format (ELL: 32 rows, a row per lane,
+ * or a slice of diagonals; SELL: the handle's work items; mode -1 and -5), a
+ * COO handle as COO chunks of 32*items entries per warp (mode -2) and a BSR
+ * handle as block rows of r lanes for each block taken at once (mode -4),
+ * unless the tuner finds a CSR mode faster; any other handle runs from its
+ * CSR arrays as nonzero chunks of 32*items entries per warp (split, mode 0)
+ * or rows with 1..32 lanes each (vector, mode = lanes per row).
+ * The kernel is captured in a CUDA graph; the warp that draws last resets the
+ * counter, so launches of one plan follow each other and never overlap.
  *
  * spmv_batch_create: hs[i] (all of one value type), alpha[i], beta[i] (host
  * arrays) and device vectors d_x[i] (n_i entries), d_y[i] (m_i entries), i <
